@@ -55,17 +55,6 @@ constexpr int engine_extra_regs() {
     return SET::R + 2 * SET::P == 53 ? 0 : (SET::P > 20 ? 24 : (SET::P > 16 ? 12 : 6));
 }
 
-// Moments, equilibrium, force and relaxation of one node (register values
-// f in place): the arithmetic of k_step_ct, shared by both engine kernels.
-template <class SET, int N, typename S, typename C>
-__device__ __forceinline__ CellCoef<C> res_collide(const KParams<C>& k, C* f) {
-    C drho, Jx = 0, Jy = 0, Kxx = 0, Kxy = 0, Kyy = 0;
-    moments_ct<SET, S, C>(k, f, drho, Jx, Jy, Kxx, Kxy, Kyy, std::make_integer_sequence<int, SET::P>{});
-    const CellCoef<C> q = cell_coef<N, C>(k, drho, Jx, Jy, Kxx, Kxy, Kyy);
-    relax_ct<SET, N, S, C>(k, q, f);
-    return q;
-}
-
 // Copy the parts of a solve's constants that kernels of a compiled set read:
 // the scalars and the first V (per plane) or P (per pair) entries of every
 // array; the arrays are sized for LBM_MAX_V, so this moves about a third of
@@ -99,8 +88,10 @@ __device__ __forceinline__ void copy_params(const KParams<C>& src, KParams<C>& d
 
 // emit: 0 = nothing, 1 = rho, u_x, u_y into the moment fields, 2 = u_x into prev
 template <class SET, int N, typename S, typename C>
-__global__ void __launch_bounds__(kBlock, min_blocks_for(SET::R + 2 * SET::P + engine_extra_regs<SET>(),
-                                                         sizeof(C)))
+__global__ void __launch_bounds__(kBlock, sizeof(C) == 8
+                                              ? (SET::P > 20 ? 3 : 4)
+                                              : min_blocks_for(SET::R + 2 * SET::P + engine_extra_regs<SET>(),
+                                                               sizeof(C)))
 k_engine_step(const EngineSolve<C>* __restrict__ solves, const EngineTile* __restrict__ tiles,
               const int* __restrict__ ntiles_p, const int* __restrict__ tile_off_p,
               int* __restrict__ counter,
@@ -175,8 +166,7 @@ k_engine_step(const EngineSolve<C>* __restrict__ solves, const EngineTile* __res
             const bool rows = !fast && ya >= k.maxey && yb < k.Ny - k.maxey;
             C f[V];
             if (fast) {
-#pragma unroll
-                for (int a = 0; a < V; ++a) f[a] = ld_val<S, C>(ld_stream(sp[a] + cell));
+                take<SET, S, C>(f, [&](auto a) { return sp[a] + cell; });
             } else if (rows || (cell / k.Nx >= k.maxey && cell / k.Nx < k.Ny - k.maxey)) {
                 // nodes away from the walls (the whole sub-tile, or this node of a wall tile)
                 pull_rows_any<SET, S, C>(k, sp, cell, f);
@@ -185,11 +175,9 @@ k_engine_step(const EngineSolve<C>* __restrict__ solves, const EngineTile* __res
                 const int x = cell - y * k.Nx;
                 pull_wall_ct<SET, S, C>(k, src, x, y, f, std::make_integer_sequence<int, V>{});
             }
-            const CellCoef<C> q = res_collide<SET, N, S, C>(k, f);
-            S out[V];
-            pack_ct<SET, S, C>(f, sr_seed<S, C>(seed + unsigned(tile.slot) * 0x632be5abu, cell), out);
-#pragma unroll
-            for (int a = 0; a < V; ++a) dp[a][cell] = out[a];
+            const CellCoef<C> q = finish_node<SET, N, S, C>(
+                k, f, emit != 0, sr_seed<S, C>(seed + unsigned(tile.slot) * 0x632be5abu, cell),
+                [&](auto a, S v) { dp[a][cell] = v; });
             if (emit == 1) {
                 B.rho[cell] = 1.0 + (double)q.drho;
                 B.ux[cell] = (double)q.ux;
@@ -251,11 +239,13 @@ __host__ __device__ constexpr int set_maxey() {
     return m;
 }
 
-// Threads of a resident block: the V populations of a node stay in
-// registers, so fp64 (two registers a value) halves the block.
+// Threads of a resident block: in fp32 the V populations of a node stay in
+// registers; fp64 reads them again (res_update64) and needs about 96 registers
+// for 16 velocities and 128 for the larger sets.
 template <class SET, typename C = float>
 __host__ __device__ constexpr int res_threads() {
-    return (SET::R + 2 * SET::P <= 16 ? 1024 : 512) / (sizeof(C) == 8 ? 2 : 1);
+    constexpr bool small = SET::R + 2 * SET::P <= 16;
+    return sizeof(C) == 8 ? (small ? 640 : 512) : (small ? 1024 : 512);
 }
 
 // (x + d) mod Nx for x in [0, Nx); mode 0: Nx = 1, 1: Nx >= |d|, 2: any Nx
@@ -322,34 +312,76 @@ __device__ __forceinline__ void res_pull_wall(const KParams<C>& k, const S* sb, 
     ((f[I] = res_wall_value<SET, S, C, STEP_A, I>(k, sb, PS, x, y, pb, pt)), ...);
 }
 
-template <class SET, typename S, typename C, int MODE, bool STEP_A, int... I>
-__device__ __forceinline__ void res_pull(const KParams<C>& k, const S* sb, int PS, int x, int y,
-                                         C* f, std::integer_sequence<int, I...>) {
+// Element, relative to the channel's planes, that a node reads population A
+// from (res_src) and writes it to (res_dst).  The slot a population is written
+// to is the slot its opposite was read from.
+template <class SET, int MODE, bool STEP_A, int A>
+__device__ __forceinline__ int res_src(int PS, int Nx, int x, int y) {
     constexpr int G = set_maxey<SET>();
-    const int Nx = k.Nx;
-    if constexpr (STEP_A) {
-        const int o = (y + G) * Nx + x;
-        ((f[I] = ld_val<S, C>(sb[I * PS + o])), ...);
-    } else {
-        ((f[I] = ld_val<S, C>(sb[plane_opp<SET>(I) * PS + (y - plane_ey<SET>(I) + G) * Nx +
-                                 xwrap<-plane_ex<SET>(I), MODE>(x, Nx)])), ...);
-    }
+    if constexpr (STEP_A) return A * PS + (y + G) * Nx + x;
+    else return plane_opp<SET>(A) * PS + (y - plane_ey<SET>(A) + G) * Nx + xwrap<-plane_ex<SET>(A), MODE>(x, Nx);
+}
+template <class SET, int MODE, bool STEP_A, int A>
+__device__ __forceinline__ int res_dst(int PS, int Nx, int x, int y) {
+    constexpr int G = set_maxey<SET>();
+    if constexpr (STEP_A) return plane_opp<SET>(A) * PS + (y + G) * Nx + x;
+    else return A * PS + (y + plane_ey<SET>(A) + G) * Nx + xwrap<plane_ex<SET>(A), MODE>(x, Nx);
 }
 
-template <class SET, typename S, typename C, int MODE, bool STEP_A, int... I>
-__device__ __forceinline__ void res_push(const KParams<C>& k, S* sb, int PS, int x, int y, const C* f,
-                                         unsigned rs, std::integer_sequence<int, I...>) {
-    constexpr int G = set_maxey<SET>();
+// Pull (away from the walls), collision and push of one node, its x wrap mode
+// known.
+template <class SET, int N, typename S, typename C, int MODE, bool STEP_A>
+__device__ __forceinline__ CellCoef<C> res_update(const KParams<C>& k, S* sb, int PS, int x, int y, bool wall,
+                                                  unsigned rs, bool want, C* f) {
+    constexpr int V = SET::R + 2 * SET::P;
     const int Nx = k.Nx;
-    S out[sizeof...(I)];
-    pack_ct<SET, S, C>(f, rs, out);
-    if constexpr (STEP_A) {
-        const int o = (y + G) * Nx + x;
-        ((sb[plane_opp<SET>(I) * PS + o] = out[I]), ...);
-    } else {
-        ((sb[I * PS + (y + plane_ey<SET>(I) + G) * Nx + xwrap<plane_ex<SET>(I), MODE>(x, Nx)] =
-              out[I]), ...);
+    if (!wall)
+        for_planes([&](auto a) {
+            f[a] = ld_val<S, C>(sb[res_src<SET, MODE, STEP_A, decltype(a)::value>(PS, Nx, x, y)]);
+        }, std::make_integer_sequence<int, V>{});
+    return finish_node<SET, N, S, C>(k, f, want, rs, [&](auto a, S v) {
+        sb[res_dst<SET, MODE, STEP_A, decltype(a)::value>(PS, Nx, x, y)] = v;
+    });
+}
+
+// The same for an fp64 node, which reads its populations where they lie: a wall
+// node first writes its wall fills into the slots they would have come from,
+// which only this node touches in this step.
+template <class SET, int N, int MODE, bool STEP_A>
+__device__ __forceinline__ CellCoef<double> res_update64(const KParams<double>& k, double* sb, int PS, int x,
+                                                         int y, bool want) {
+    constexpr int G = set_maxey<SET>();
+    const int Nx = MODE == 0 ? 1 : k.Nx, o = (y + G) * Nx + x;
+    // node (x + dx, y + dy) in plane coordinates, x periodic
+    auto at = [&](int dx, int dy) {
+        if constexpr (MODE == 0) return o + dy;
+        int t = x + dx;
+        if constexpr (MODE == 1) {
+            t += t < 0 ? Nx : 0;
+            t -= t >= Nx ? Nx : 0;
+        } else {
+            t %= Nx;
+            t += t < 0 ? Nx : 0;
+        }
+        return (y + dy + G) * Nx + t;
+    };
+    auto get = [&](int a, int opp, int ex, int ey) -> double& {
+        return STEP_A ? sb[a * PS + o] : sb[opp * PS + at(-ex, -ey)];
+    };
+    if (y < G || y >= k.Ny - G) {
+        const double pb = y < G ? res_wall_dpsi<SET, double, double, true, STEP_A>(k, sb, PS, x) : 0.0;
+        const double pt = y >= k.Ny - G ? res_wall_dpsi<SET, double, double, false, STEP_A>(k, sb, PS, x) : 0.0;
+#pragma unroll 1
+        for (int a = 0; a < k.V; ++a) {
+            const int ys = y - k.ey[a];
+            if (ys < 0 || ys >= k.Ny)
+                get(a, a < k.R ? a : (a < k.R + k.P ? a + k.P : a - k.P), k.ex[a], k.ey[a]) =
+                    mul_rn(ys < 0 ? pb : pt, k.cw[a]);
+        }
     }
+    return collide64<SET, N>(k, want, get, [&](int a, int opp, int ex, int ey, double v) {
+        (STEP_A ? sb[opp * PS + o] : sb[a * PS + at(ex, ey)]) = v;
+    });
 }
 
 template <typename C>
@@ -375,26 +407,23 @@ __device__ __forceinline__ void res_node(const EngineSolve<C>& B, S* sb, int PS,
     const int Nx = k.Nx, Ny = k.Ny;
     const int y = Nx == 1 ? cell : cell / Nx;     // one-column channels need no division
     const int x = cell - y * Nx;
-    C f[V];
-    const int mode = Nx == 1 ? 0 : (Nx >= k.maxex ? 1 : 2);
-    if (y >= G && y < Ny - G) {
-        if (mode == 0)
-            res_pull<SET, S, C, 0, STEP_A>(k, sb, PS, x, y, f, std::make_integer_sequence<int, V>{});
-        else if (mode == 1)
-            res_pull<SET, S, C, 1, STEP_A>(k, sb, PS, x, y, f, std::make_integer_sequence<int, V>{});
-        else
-            res_pull<SET, S, C, 2, STEP_A>(k, sb, PS, x, y, f, std::make_integer_sequence<int, V>{});
+    CellCoef<C> q;
+    if constexpr (sizeof(C) == 8) {
+        if (Nx == 1) q = res_update64<SET, N, 0, STEP_A>(k, sb, PS, x, y, emit != 0);
+        else if (Nx >= k.maxex) q = res_update64<SET, N, 1, STEP_A>(k, sb, PS, x, y, emit != 0);
+        else q = res_update64<SET, N, 2, STEP_A>(k, sb, PS, x, y, emit != 0);
     } else {
-        res_pull_wall<SET, S, C, STEP_A>(k, sb, PS, x, y, f, std::make_integer_sequence<int, V>{});
+        C f[V];
+        const bool wall = y < G || y >= Ny - G;
+        if (wall) res_pull_wall<SET, S, C, STEP_A>(k, sb, PS, x, y, f, std::make_integer_sequence<int, V>{});
+        const unsigned rs = sr_seed<S, C>(seed + unsigned(slot) * 0x632be5abu, cell);
+        if (Nx == 1)
+            q = res_update<SET, N, S, C, 0, STEP_A>(k, sb, PS, x, y, wall, rs, emit != 0, f);
+        else if (Nx >= k.maxex)
+            q = res_update<SET, N, S, C, 1, STEP_A>(k, sb, PS, x, y, wall, rs, emit != 0, f);
+        else
+            q = res_update<SET, N, S, C, 2, STEP_A>(k, sb, PS, x, y, wall, rs, emit != 0, f);
     }
-    const CellCoef<C> q = res_collide<SET, N, S, C>(k, f);
-    const unsigned rs = sr_seed<S, C>(seed + unsigned(slot) * 0x632be5abu, cell);
-    if (mode == 0)
-        res_push<SET, S, C, 0, STEP_A>(k, sb, PS, x, y, f, rs, std::make_integer_sequence<int, V>{});
-    else if (mode == 1)
-        res_push<SET, S, C, 1, STEP_A>(k, sb, PS, x, y, f, rs, std::make_integer_sequence<int, V>{});
-    else
-        res_push<SET, S, C, 2, STEP_A>(k, sb, PS, x, y, f, rs, std::make_integer_sequence<int, V>{});
     res_emit<C>(B, q, cell, emit);
 }
 
@@ -409,7 +438,7 @@ k_engine_resident(const EngineSolve<C>* __restrict__ solves, const ResBundle* __
                   const unsigned* __restrict__ seed_p, int K) {
     constexpr int R = SET::R, P = SET::P, V = R + 2 * P, G = set_maxey<SET>();
     constexpr int BT = res_threads<SET, C>();
-    constexpr int NPT = kResNodes / BT;
+    constexpr int NPT = (kResNodes + BT - 1) / BT;
     extern __shared__ __align__(16) unsigned char res_smem[];
     S* const sm = reinterpret_cast<S*>(res_smem);
     __shared__ ResChannel sch[kResMaxCh];

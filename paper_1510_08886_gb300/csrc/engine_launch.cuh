@@ -28,7 +28,7 @@ struct EngineLaunch {
 template <class SET, int N, typename S>
 cudaError_t engine_step_one(const EngineLaunch& L, cudaStream_t st) {
     using C = CompOf<S>;
-    k_engine_step<SET, N, S, C><<<L.grid, kBlock, 0, st>>>(
+    k_engine_step<SET, N, S, C><<<L.grid, kBlock, step_smem<SET, C>(), st>>>(
         static_cast<const EngineSolve<C>*>(L.solves), L.tiles, L.ntiles, L.tile_off, L.counter, L.seed,
         L.parity, L.emit, L.chunk, L.lm);
     return cudaGetLastError();
@@ -145,8 +145,17 @@ int engine_resident_attr_t(int set_id, int N, size_t smem) {
 // resident blocks per SM of the engine kernel of (set, N)
 template <class SET, int N, typename S>
 int engine_occ_one() {
+    // fp64: opt into the scratch as well (the engine asks for the occupancy of a
+    // group before it captures its launches)
+    constexpr int smem = step_smem<SET, CompOf<S>>();
     int b = 0;
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_engine_step<SET, N, S, CompOf<S>>, kBlock, 0);
+    if ((smem && cudaFuncSetAttribute(k_engine_step<SET, N, S, CompOf<S>>,
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_engine_step<SET, N, S, CompOf<S>>, kBlock, smem) !=
+            cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
     return b;
 }
 

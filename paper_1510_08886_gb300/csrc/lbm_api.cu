@@ -87,9 +87,10 @@ struct CompiledSet {
     int R, P;
     const int* ex;
     const int* ey;
+    lbm::fx::SetInfo fx;
 };
 template <class SET>
-constexpr CompiledSet compiled() { return {SET::R, SET::P, SET::ex, SET::ey}; }
+constexpr CompiledSet compiled() { return {SET::R, SET::P, SET::ex, SET::ey, lbm::fx::set_info<SET>()}; }
 const CompiledSet kSets[] = {compiled<lbm::SetD2V16>(), compiled<lbm::SetD2V32>(),
                              compiled<lbm::SetD2V33>(), compiled<lbm::SetD2V53>(),
                              compiled<lbm::SetD2V40>(), compiled<lbm::SetD2V48>()};
@@ -243,6 +244,9 @@ void fill_params_impl(const lbm::SolveSpec* s, KParams<C>& k) {
     k.htc2 = k.half_tau * k.c2;
     k.tc = k.tau * k.c;
     k.cg = k.c * k.gx;
+    if constexpr (sizeof(C) == 8)
+        if (s->set_id >= 0) k.fx = lbm::fx::make_consts(s->c, s->tau, s->dt, s->g, s->R, s->P, s->ex.data(), s->ey.data(),
+                                        s->w.data(), kSets[s->set_id].fx);
 }
 
 int cuda_status(cudaError_t e) {
@@ -611,6 +615,15 @@ int create_common(const lbm_dvm* dvm, int order, int Nx, int Ny, double Kn, doub
     s->b.status = reinterpret_cast<unsigned*>(base + L.status);
     lbm::fill_params(*s, s->k64);
     lbm::fill_params(*s, s->k32);
+    if (precision == LBM_FP64 && !lbm::warp_path_lanes(s->P, (long long)Nx * Ny)) {
+        const cudaError_t e = lbm::allow_step_scratch_fp64(s->set_id, s->N);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            if (s->owns) cudaFree(s->ws);
+            delete s;
+            return cuda_status(e);
+        }
+    }
     if (precision == LBM_FP64 || precision == LBM_FP32) {
         const int LP = lbm::warp_path_lanes(s->P, (long long)Nx * Ny);
         if (LP && precision == LBM_FP64) lbm::plan_cluster(s->k64, s->N, LP, s->cl);

@@ -7,6 +7,7 @@
 
 #include <vector>
 
+#include "fx64.cuh"
 #include "lbm.h"
 
 namespace lbm {
@@ -26,6 +27,11 @@ constexpr int min_blocks_for(int V, int bytes) {
 }
 constexpr int kReduceBlocks = 304;   // 2 x 152 SMs for the partial sums
 constexpr int kReduceThreads = 256;
+
+// Constants of the fixed-point collision: fp64 solves only.
+struct NoFx {};
+template <typename C> struct FxOf { using type = NoFx; };
+template <> struct FxOf<double> { using type = fx::Consts; };
 
 // Per-solve constants, passed by value to every kernel (__grid_constant__).
 // Planes are in the solver's internal order: R rest planes (R = 0 or 1),
@@ -77,6 +83,7 @@ struct KParams {
     // products of constants (formed on the host in C, as the device would):
     // hdt gx, hdt gy, two_tau gx, two_tau gy, two_tau c2, half_tau c2, tau c, c gx
     C hdt_gx, hdt_gy, tgx, tgy, ttc2, htc2, tc, cg;
+    typename FxOf<C>::type fx;
 };
 
 // Device buffers of one solver.
@@ -95,6 +102,8 @@ struct DevBufs {
 // Return cudaSuccess or the launch error.
 cudaError_t launch_step_fp64(const KParams<double>& k, int N, const void* src,
                              void* dst, const DevBufs& b, cudaStream_t st);
+// once per solver, before its first step
+cudaError_t allow_step_scratch_fp64(int set_id, int N);
 cudaError_t launch_init_fp64(const KParams<double>& k, int N, const double* rho0,
                              void* dst, const DevBufs& b, cudaStream_t st);
 cudaError_t launch_step_fp32(const KParams<float>& k, int N, const void* src,

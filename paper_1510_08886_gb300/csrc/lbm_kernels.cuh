@@ -466,14 +466,6 @@ __device__ __forceinline__ C wall_value(const KParams<C>& k, const S* __restrict
     return ld_val<S, C>(src[(long long)A * k.plane + (long long)ys * k.Nx + xs]);
 }
 
-template <class SET, typename S, typename C, int... I>
-__device__ __forceinline__ void pull_wall_ct(const KParams<C>& k, const S* __restrict__ src, int x,
-                                             int y, C* f, std::integer_sequence<int, I...>) {
-    const C pb = y < k.maxey ? C(wall_dpsi_ct<SET, S, C, true>(k, src, x)) : C(0);
-    const C pt = y >= k.Ny - k.maxey ? C(wall_dpsi_ct<SET, S, C, false>(k, src, x)) : C(0);
-    ((f[I] = wall_value<SET, S, C, I>(k, src, x, y, pb, pt)), ...);
-}
-
 // e_y of plane a of a compiled set (rest, the P pair members, their negatives)
 template <class SET>
 __host__ __device__ constexpr int plane_ey_ct(int a) {
@@ -795,6 +787,85 @@ __device__ __forceinline__ void relax_ct(const KParams<C>& k, const CellCoef<C>&
     }
 }
 
+// FP64 collision of one node with run-time loops over the pairs: what a node
+// outside the range of the fixed-point form takes.
+template <int N, class GET, class PUT>
+__device__ __forceinline__ CellCoef<double> slow_collide(const KParams<double>& k, const GET& get,
+                                                         const PUT& put) {
+    const int R = k.R, P = k.P;
+    double drho = R ? get(0, 0, 0, 0) : 0.0, Jx = 0, Jy = 0, Kxx = 0, Kxy = 0, Kyy = 0;
+#pragma unroll 1
+    for (int p = 0; p < P; ++p) {
+        const int a = R + p, b = R + P + p, x = k.ex[a], y = k.ey[a];
+        const double fp = get(a, b, x, y), fm = get(b, a, -x, -y);
+        const double sum = fp + fm, dif = fp - fm;
+        drho += sum;
+        Jx = fma(k.pex[p], dif, Jx);
+        Jy = fma(k.pey[p], dif, Jy);
+        Kxx = fma(k.pexx[p], sum, Kxx);
+        Kxy = fma(k.pexy2[p], sum, Kxy);
+        Kyy = fma(k.peyy[p], sum, Kyy);
+    }
+    const CellCoef<double> q = cell_coef<N, double>(k, drho, Jx, Jy, Kxx, 0.5 * Kxy, Kyy);
+    if (R) put(0, 0, 0, 0, fma(k.one_m_omega, get(0, 0, 0, 0), k.omw_rest * q.a0));
+#pragma unroll 1
+    for (int p = 0; p < P; ++p) {
+        const int a = R + p, b = R + P + p, x = k.ex[a], y = k.ey[a];
+        double fp = get(a, b, x, y), fm = get(b, a, -x, -y);
+        if (k.force) pair_update<true, double>(k, q, p, fp, fm);
+        else pair_update<false, double>(k, q, p, fp, fm);
+        put(a, b, x, y, fp);
+        put(b, a, -x, -y, fm);
+    }
+    return q;
+}
+
+// A plane index known at compile time, and fn(Plane) for every plane.
+template <int A>
+struct Plane {
+    static constexpr int value = A;
+    __host__ __device__ constexpr operator int() const { return A; }
+};
+template <class FN, int... I>
+__device__ __forceinline__ void for_planes(const FN& fn, std::integer_sequence<int, I...>) {
+    (fn(Plane<I>{}), ...);
+}
+
+// fp64 collision of a node of a compiled set (get, put: see fx::collide).  The
+// moments rho, u of the result are valid when want is set; drho and rho are
+// always fit for flag_density.
+template <class SET, int N, class GET, class PUT>
+__device__ __forceinline__ CellCoef<double> collide64(const KParams<double>& k, bool want, const GET& get,
+                                                      const PUT& put) {
+    fx::Sums m;
+    int E;
+    const bool done = k.force ? fx::collide<SET, N, true>(k.fx, k.one_m_omega, m, E, get, put)
+                              : fx::collide<SET, N, false>(k.fx, k.one_m_omega, m, E, get, put);
+    if (!done) return slow_collide<N>(k, get, put);
+    CellCoef<double> q;
+    q.drho = 0.0;
+    q.rho = 1.0;
+    if (want) {
+        // sums times 2^(E - 1075 - S0), in two exact steps
+        const double u = __hiloint2double((E + 1 - fx::guard_bits<SET>()) << 20, 0);
+        auto val = [&](long long v) { return mul_rn(mul_rn(double(v), 0x1p-53), u); };
+        q.drho = val(m.d);
+        q.rho = 1.0 + q.drho;
+        const double inv = 1.0 / q.rho;
+        q.ux = fma(mul_rn(k.c, val(m.jx)), inv, k.hdt_gx);
+        q.uy = fma(mul_rn(k.c, val(m.jy)), inv, k.hdt_gy);
+    }
+    return q;
+}
+
+// Per-thread scratch of the fp64 step kernels: a block's populations in
+// dynamic shared memory ([V][kBlock]), so that they need not stay in registers
+// between the sums and the relaxation.
+template <class SET, typename C>
+__host__ __device__ constexpr int step_smem() {
+    return sizeof(C) == 8 ? (SET::R + 2 * SET::P) * kBlock * 8 : 0;
+}
+
 // Stored values of a node's post-collision register values.  16-bit storage
 // rounds stochastically, two values per conversion: the rest value with a
 // zero partner, then each +-e pair, with the random bits r0 + (p + 1) phi
@@ -818,19 +889,95 @@ __device__ __forceinline__ void pack_ct(const C* f, unsigned r0, S* out) {
     }
 }
 
-// Middle path of a tile whose rows all lie at least max|e_y| rows from both
-// walls (the nodes may wrap around x): the source of plane a is
-// cell - off[a] + dx[a] (+ Nx when x - e_x wraps below 0), with
-// sp[a] = lattice + a plane - off[a].
-template <int V, typename S, typename C, typename PTR>
-__device__ __forceinline__ void pull_rows(const KParams<C>& k, const PTR& sp, int cell, C* f) {
-    const int y = cell / k.Nx;
-    const int x = cell - y * k.Nx;
-#pragma unroll
-    for (int a = 0; a < V; ++a) {
-        const int i = cell + k.dx[a] + (x < k.sx[a] ? k.Nx : 0);
-        f[a] = ld_val<S, C>(static_cast<const S*>(sp[a])[i]);
+// This thread's column of the block's scratch: population a at [a * kBlock].
+__device__ __forceinline__ double* step_scratch() {
+    extern __shared__ __align__(16) unsigned char step_scratch_raw[];
+    return reinterpret_cast<double*>(step_scratch_raw) + threadIdx.x;
+}
+
+// Copy one population to the scratch without passing a register.
+__device__ __forceinline__ void copy_async(double* dst, const double* src) {
+    const unsigned d = unsigned(__cvta_generic_to_shared(dst));
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copies_done() {      // this thread's own copies
+    asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
+// Take a node's streamed populations: load(a) = address of the source of plane
+// a.  fp32 and 16-bit populations go to registers f, fp64 ones to the scratch.
+template <class SET, typename S, typename C, class SRC>
+__device__ __forceinline__ void take(C* f, const SRC& load) {
+    constexpr auto planes = std::make_integer_sequence<int, SET::R + 2 * SET::P>{};
+    if constexpr (sizeof(C) == 8) {
+        double* sf = step_scratch();
+        for_planes([&](auto a) { copy_async(sf + a * kBlock, load(a)); }, planes);
+    } else {
+        for_planes([&](auto a) { f[a] = ld_val<S, C>(ld_stream(load(a))); }, planes);
     }
+}
+
+// Collision of a node of a compiled set with streamed values f (fp64: the
+// scratch), its new values handed to put(a, value) in storage form; r0 the
+// node's hash for 16-bit stores.
+template <class SET, int N, typename S, typename C, class PUT>
+__device__ __forceinline__ CellCoef<C> finish_node(const KParams<C>& k, C* f, bool want, unsigned r0,
+                                                   const PUT& put) {
+    constexpr int V = SET::R + 2 * SET::P;
+    if constexpr (sizeof(C) == 8) {
+        const double* sf = step_scratch();
+        copies_done();
+        return collide64<SET, N>(k, want, [&](int a, int, int, int) { return sf[a * kBlock]; },
+                                 [&](int a, int, int, int, double v) { put(a, v); });
+    } else {
+        C drho, Jx = 0, Jy = 0, Kxx = 0, Kxy = 0, Kyy = 0;
+        moments_ct<SET, S, C>(k, f, drho, Jx, Jy, Kxx, Kxy, Kyy, std::make_integer_sequence<int, SET::P>{});
+        const CellCoef<C> q = cell_coef<N, C>(k, drho, Jx, Jy, Kxx, Kxy, Kyy);
+        relax_ct<SET, N, S, C>(k, q, f);
+        S out[V];
+        pack_ct<SET, S, C>(f, r0, out);
+        for_planes([&](auto a) { put(a, out[a]); }, std::make_integer_sequence<int, V>{});
+        return q;
+    }
+}
+
+// fp64: the populations of a node near a wall into the scratch, the walls'
+// dPsi given (pb bottom, pt top; 0 where out of reach): the fill where the
+// source lies beyond a wall, the pull otherwise.
+__device__ __forceinline__ void take_wall64(const KParams<double>& k, const double* __restrict__ src, int x,
+                                            int y, double pb, double pt) {
+    double* sf = step_scratch();
+#pragma unroll 4
+    for (int a = 0; a < k.V; ++a) {
+        const int ys = y - k.ey[a];
+        if (ys < 0 || ys >= k.Ny) {
+            sf[a * kBlock] = mul_rn(ys < 0 ? pb : pt, k.cw[a]);
+            continue;
+        }
+        int xs = x - k.sx[a];
+        xs += (xs < 0) ? k.Nx : 0;
+        copy_async(sf + a * kBlock, src + (long long)a * k.plane + (long long)ys * k.Nx + xs);
+    }
+}
+
+// Populations of a wall node of a compiled set (registers f; fp64: the scratch).
+template <class SET, typename S, typename C, int... I>
+__device__ __forceinline__ void pull_wall_ct(const KParams<C>& k, const S* __restrict__ src, int x,
+                                             int y, C* f, std::integer_sequence<int, I...>) {
+    const C pb = y < k.maxey ? C(wall_dpsi_ct<SET, S, C, true>(k, src, x)) : C(0);
+    const C pt = y >= k.Ny - k.maxey ? C(wall_dpsi_ct<SET, S, C, false>(k, src, x)) : C(0);
+    if constexpr (sizeof(C) == 8) take_wall64(k, src, x, y, pb, pt);
+    else ((f[I] = wall_value<SET, S, C, I>(k, src, x, y, pb, pt)), ...);
+}
+
+// Resident blocks per SM asked of the compiler for k_step_ct.  fp64: 96
+// registers hold the fixed-point collision without spills (D2V33 4096 x 512, us
+// per step at 4 / 5 / 6 blocks: 353 / 334 / 355); the scratch allows 4 for the
+// 53-velocity set.
+template <class SET, typename C>
+__host__ __device__ constexpr int step_blocks() {
+    constexpr int V = SET::R + 2 * SET::P;
+    return sizeof(C) == 8 ? 5 : min_blocks_for(V, sizeof(C));
 }
 
 // e_x of plane a of a compiled set (rest, the P pair members, their negatives)
@@ -839,51 +986,35 @@ __host__ __device__ constexpr int plane_ex(int a) {
     return a < SET::R ? 0 : (a < SET::R + SET::P ? SET::ex[a - SET::R] : -SET::ex[a - SET::R - SET::P]);
 }
 
-// Rows path with e_x known at compile time (all rows of the node away from the
-// walls).  sp[a] = lattice + a plane - (e_y Nx + e_x) (a pointer, or for the
-// single-solve kernel a byte address).  With Nx >= max|e_x|
-// the x wrap is one compare against a constant; with Nx = 1 every source lies
-// in the same column and the pull is cell + e_x.
-template <class SET, typename S, typename C, int A, class PTR>
-__device__ __forceinline__ C pull_col(const KParams<C>& k, const PTR& sp, int cell, int x,
-                                      int Nx) {
-    constexpr int EX = plane_ex<SET>(A);
-    int i;
-    if constexpr (EX == 0) {
-        i = cell;
-    } else if constexpr (EX > 0) {
-        i = cell + (x < EX ? Nx : 0);
-    } else {
-        i = cell + (x < Nx + EX ? 0 : -Nx);
-    }
-    return ld_val<S, C>(ld_stream(static_cast<const S*>(sp[A]) + i));
-}
-
-template <class SET, typename S, typename C, int A, class PTR>
-__device__ __forceinline__ C pull_col1(const KParams<C>& k, const PTR& sp, int cell) {
-    return ld_val<S, C>(ld_stream(static_cast<const S*>(sp[A]) + cell + plane_ex<SET>(A)));
-}
-
-template <class SET, typename S, typename C, class PTR, int... I>
-__device__ __forceinline__ void pull_rows_ct(const KParams<C>& k, const PTR& sp, int cell,
-                                             C* f, std::integer_sequence<int, I...>) {
-    const int Nx = k.Nx;
-    if (Nx == 1) {
-        ((f[I] = pull_col1<SET, S, C, I, PTR>(k, sp, cell)), ...);
-    } else {
-        const int x = cell % Nx;
-        ((f[I] = pull_col<SET, S, C, I, PTR>(k, sp, cell, x, Nx)), ...);
-    }
-}
-
-// Rows-path pull of a compiled set: the compile-time forms where they apply.
+// Rows path: all rows of the node lie at least max|e_y| rows from both walls
+// (the node may wrap around x).  sp[a] = lattice + a plane - (e_y Nx + e_x) (a
+// pointer, or for the single-solve kernel a byte address).  e_x is known at
+// compile time: with Nx >= max|e_x| the x wrap is one compare against a
+// constant, with Nx = 1 every source lies in the same column and the pull is
+// cell + e_x; narrower channels take the source from the solve's constants,
+// cell - off[a] + dx[a] (+ Nx when x - e_x wraps below 0).
 template <class SET, typename S, typename C, class PTR>
 __device__ __forceinline__ void pull_rows_any(const KParams<C>& k, const PTR& sp, int cell, C* f) {
-    constexpr int V = SET::R + 2 * SET::P;
-    if (k.Nx == 1 || k.Nx >= k.maxex)
-        pull_rows_ct<SET, S, C>(k, sp, cell, f, std::make_integer_sequence<int, V>{});
-    else
-        pull_rows<V, S, C>(k, sp, cell, f);
+    const int Nx = k.Nx;
+    if (Nx == 1) {
+        take<SET, S, C>(f, [&](auto a) {
+            return static_cast<const S*>(sp[a]) + cell + plane_ex<SET>(decltype(a)::value);
+        });
+    } else if (Nx >= k.maxex) {
+        const int x = cell % Nx;
+        take<SET, S, C>(f, [&](auto a) {
+            constexpr int EX = plane_ex<SET>(decltype(a)::value);
+            int i = cell;
+            if constexpr (EX > 0) i += x < EX ? Nx : 0;
+            else if constexpr (EX < 0) i += x < Nx + EX ? 0 : -Nx;
+            return static_cast<const S*>(sp[a]) + i;
+        });
+    } else {
+        const int x = cell % Nx;
+        take<SET, S, C>(f, [&](auto a) {
+            return static_cast<const S*>(sp[a]) + (cell + k.dx[a] + (x < k.sx[a] ? Nx : 0));
+        });
+    }
 }
 
 // ---- wall strips ------------------------------------------------------------
@@ -943,15 +1074,10 @@ __device__ __forceinline__ void wall_strip(const KParams<C>& k, const S* __restr
     const C dpsi = C(((part[0][lane] + part[1][lane]) + (part[2][lane] + part[3][lane])) * k.inv_den);
     const int cell = y * k.Nx + x;
     C f[V];
-    strip_values<SET, S, C, BOTTOM>(k, src, x, y, dpsi, f, seq);
-    C drho, Jx = 0, Jy = 0, Kxx = 0, Kxy = 0, Kyy = 0;
-    moments_ct<SET, S, C>(k, f, drho, Jx, Jy, Kxx, Kxy, Kyy, std::make_integer_sequence<int, P>{});
-    const CellCoef<C> q = cell_coef<N, C>(k, drho, Jx, Jy, Kxx, Kxy, Kyy);
-    relax_ct<SET, N, S, C>(k, q, f);
-    S out[V];
-    pack_ct<SET, S, C>(f, sr_seed<S, C>(k.seed, cell), out);
-#pragma unroll
-    for (int a = 0; a < V; ++a) static_cast<S*>(k.dstp[a])[cell] = out[a];
+    if constexpr (sizeof(C) == 8) take_wall64(k, src, x, y, dpsi, dpsi);
+    else strip_values<SET, S, C, BOTTOM>(k, src, x, y, dpsi, f, seq);
+    const CellCoef<C> q = finish_node<SET, N, S, C>(k, f, k.emit != 0, sr_seed<S, C>(k.seed, cell),
+                                                    [&](auto a, S v) { static_cast<S*>(k.dstp[a])[cell] = v; });
     emit_moments<C>(k, q, cell, b);
     flag_density<C>(q, b.status);
 }
@@ -966,7 +1092,7 @@ __device__ __forceinline__ void wall_strip(const KParams<C>& k, const S* __restr
 //    select per population;
 //  - general path: periodic wrap in x and the diffuse-wall fill near walls.
 template <class SET, int N, typename S, typename C>
-__global__ void __launch_bounds__(kBlock, min_blocks_for(SET::R + 2 * SET::P, sizeof(C)))
+__global__ void __launch_bounds__(kBlock, step_blocks<SET, C>())
 k_step_ct(const __grid_constant__ KParams<C> k, const S* __restrict__ src, S* __restrict__ dst,
           const DevBufs b) {
     constexpr int R = SET::R, P = SET::P, V = R + 2 * P;
@@ -1002,8 +1128,7 @@ k_step_ct(const __grid_constant__ KParams<C> k, const S* __restrict__ src, S* __
     }
     C f[V];
     if (wfast) {
-#pragma unroll
-        for (int a = 0; a < V; ++a) f[a] = ld_val<S, C>(ld_stream(static_cast<const S*>(k.srcf[a]) + cell));
+        take<SET, S, C>(f, [&](auto a) { return static_cast<const S*>(k.srcf[a]) + cell; });
     } else if (rows) {
         if (cell >= k.ncell) return;
         pull_rows_any<SET, S, C>(k, k.srcf, cell, f);
@@ -1017,14 +1142,8 @@ k_step_ct(const __grid_constant__ KParams<C> k, const S* __restrict__ src, S* __
         else
             pull_wall_ct<SET, S, C>(k, src, x, y, f, std::make_integer_sequence<int, V>{});
     }
-    C drho, Jx = 0, Jy = 0, Kxx = 0, Kxy = 0, Kyy = 0;
-    moments_ct<SET, S, C>(k, f, drho, Jx, Jy, Kxx, Kxy, Kyy, std::make_integer_sequence<int, P>{});
-    const CellCoef<C> q = cell_coef<N, C>(k, drho, Jx, Jy, Kxx, Kxy, Kyy);
-    relax_ct<SET, N, S, C>(k, q, f);
-    S out[V];
-    pack_ct<SET, S, C>(f, sr_seed<S, C>(k.seed, cell), out);
-#pragma unroll
-    for (int a = 0; a < V; ++a) static_cast<S*>(k.dstp[a])[cell] = out[a];
+    const CellCoef<C> q = finish_node<SET, N, S, C>(k, f, k.emit != 0, sr_seed<S, C>(k.seed, cell),
+                                                    [&](auto a, S v) { static_cast<S*>(k.dstp[a])[cell] = v; });
     emit_moments<C>(k, q, cell, b);
     flag_density<C>(q, b.status);
 }
@@ -1236,6 +1355,7 @@ template <int N, typename S, typename C>
 cudaError_t launch_step_n(const KParams<C>& k, const S* src, S* dst, const DevBufs& b,
                           cudaStream_t st) {
     const dim3 g = grid_for(k);
+#define LBM_STEP(SET) k_step_ct<SET, N, S, C><<<g, kBlock, step_smem<SET, C>(), st>>>(k, src, dst, b)
     // fp64 and fp32 channels too small to fill the GPU with one node per
     // thread: several lanes per node (k_step_warp) spread the work over more
     // SMs, and the same body runs resident chunks on a cluster (k_cluster.cu)
@@ -1244,15 +1364,30 @@ cudaError_t launch_step_n(const KParams<C>& k, const S* src, S* dst, const DevBu
         if (LP) return launch_warp<N, S, C>(k, LP, src, dst, b, st);
     }
     switch (k.set_id) {
-        case 0: k_step_ct<SetD2V16, N, S, C><<<g, kBlock, 0, st>>>(k, src, dst, b); break;
-        case 1: k_step_ct<SetD2V32, N, S, C><<<g, kBlock, 0, st>>>(k, src, dst, b); break;
-        case 2: k_step_ct<SetD2V33, N, S, C><<<g, kBlock, 0, st>>>(k, src, dst, b); break;
-        case 3: k_step_ct<SetD2V53, N, S, C><<<g, kBlock, 0, st>>>(k, src, dst, b); break;
-        case 4: k_step_ct<SetD2V40, N, S, C><<<g, kBlock, 0, st>>>(k, src, dst, b); break;
-        case 5: k_step_ct<SetD2V48, N, S, C><<<g, kBlock, 0, st>>>(k, src, dst, b); break;
+        case 0: LBM_STEP(SetD2V16); break;
+        case 1: LBM_STEP(SetD2V32); break;
+        case 2: LBM_STEP(SetD2V33); break;
+        case 3: LBM_STEP(SetD2V53); break;
+        case 4: LBM_STEP(SetD2V40); break;
+        case 5: LBM_STEP(SetD2V48); break;
         default: k_generic<N, false, S, C><<<g, kBlock, 0, st>>>(k, src, nullptr, dst, b);
     }
+#undef LBM_STEP
     return cudaGetLastError();
+}
+
+// Opt the fp64 step kernel of (set, N) into its shared-memory scratch (above
+// the 48 KB default for the larger sets).
+template <class SET>
+cudaError_t allow_scratch_n(int N) {
+    const int bytes = step_smem<SET, double>();
+    const auto a = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    switch (N) {
+        case 2: return cudaFuncSetAttribute(k_step_ct<SET, 2, double, double>, a, bytes);
+        case 3: return cudaFuncSetAttribute(k_step_ct<SET, 3, double, double>, a, bytes);
+        case 4: return cudaFuncSetAttribute(k_step_ct<SET, 4, double, double>, a, bytes);
+        default: return cudaErrorInvalidValue;
+    }
 }
 
 template <typename S, typename C>
