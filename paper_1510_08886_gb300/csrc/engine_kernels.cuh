@@ -55,35 +55,12 @@ constexpr int engine_extra_regs() {
     return SET::R + 2 * SET::P == 53 ? 0 : (SET::P > 20 ? 24 : (SET::P > 16 ? 12 : 6));
 }
 
-// Copy the parts of a solve's constants that kernels of a compiled set read:
-// the scalars and the first V (per plane) or P (per pair) entries of every
-// array; the arrays are sized for LBM_MAX_V, so this moves about a third of
-// the record.
-template <class SET, typename C>
-__device__ __forceinline__ void copy_params(const KParams<C>& src, KParams<C>& dst) {
-    using K = KParams<C>;
-    constexpr int V = SET::R + 2 * SET::P, P = SET::P;
-    constexpr int cv = int(sizeof(C) / 4) * V, cp = int(sizeof(C) / 4) * P;
-    // (first 4-byte word, words)
-    constexpr int seg[][2] = {
-        {0, int(offsetof(K, ex) / 4)},
-        {int(offsetof(K, ex) / 4), V}, {int(offsetof(K, ey) / 4), V}, {int(offsetof(K, sx) / 4), V},
-        {int(offsetof(K, off) / 4), V}, {int(offsetof(K, dx) / 4), V},
-        {int(offsetof(K, srcf) / 4), 2 * V}, {int(offsetof(K, dstp) / 4), 2 * V},
-        {int(offsetof(K, w) / 4), 2 * V},
-        {int(offsetof(K, cw) / 4), cv}, {int(offsetof(K, sw) / 4), cv}, {int(offsetof(K, isw) / 4), cv},
-        {int(offsetof(K, hw) / 4), cp}, {int(offsetof(K, hwx) / 4), cp}, {int(offsetof(K, hwy) / 4), cp},
-        {int(offsetof(K, hwxx) / 4), cp}, {int(offsetof(K, hwxy) / 4), cp}, {int(offsetof(K, hwyy) / 4), cp},
-        {int(offsetof(K, hw_rest) / 4), int((offsetof(K, pex) - offsetof(K, hw_rest)) / 4)},
-        {int(offsetof(K, pex) / 4), cp}, {int(offsetof(K, pey) / 4), cp}, {int(offsetof(K, pexx) / 4), cp},
-        {int(offsetof(K, pexy2) / 4), cp}, {int(offsetof(K, peyy) / 4), cp}, {int(offsetof(K, pge) / 4), cp},
-        {int(offsetof(K, pomw) / 4), cp},
-        {int(offsetof(K, omw_rest) / 4), int((sizeof(K) - offsetof(K, omw_rest)) / 4)}};
-    const int* s = reinterpret_cast<const int*>(&src);
-    int* d = reinterpret_cast<int*>(&dst);
-#pragma unroll
-    for (int g = 0; g < int(sizeof(seg) / sizeof(seg[0])); ++g)
-        for (int i = int(threadIdx.x); i < seg[g][1]; i += kBlock) d[seg[g][0] + i] = s[seg[g][0] + i];
+// Copy the constants of a solve that a kernel of its set reads, by the whole block.
+template <class SET, typename C, int MD>
+__device__ __forceinline__ void copy_params(const KParams<C>& src, KParams<C, MD>& dst) {
+    copy_params_by<SET::R + 2 * SET::P>(src, dst, [](int* d, const int* s, int words) {
+        for (int i = int(threadIdx.x); i < words; i += kBlock) d[i] = s[i];
+    });
 }
 
 // emit: 0 = nothing, 1 = rho, u_x, u_y into the moment fields, 2 = u_x into prev
@@ -100,7 +77,8 @@ k_engine_step(const EngineSolve<C>* __restrict__ solves, const EngineTile* __res
     __shared__ const S* sp[V];
     __shared__ S* dp[V];
     __shared__ int s_first[2];
-    __shared__ KParams<C> s_k;
+    using Rec = KParams<C, sizeof(C) == 8 ? V : LBM_MAX_V>;
+    __shared__ Rec s_k;
     const int ntiles = *ntiles_p;
     tiles += *tile_off_p;
     const unsigned seed = *seed_p + unsigned(parity);
@@ -119,13 +97,13 @@ k_engine_step(const EngineSolve<C>* __restrict__ solves, const EngineTile* __res
             const EngineTile tile = tiles[u >> lm];
             const int j = u & ((1 << lm) - 1);
             const EngineSolve<C>& B = solves[tile.slot];
-            const KParams<C>& k = s_k;
+            const Rec& k = s_k;
             if (tile.slot != cur_slot) {
                 // The previous slot's constants and plane bases are free once
                 // every thread is past its last sub-tile: at the grab's
                 // barrier for the grab's first sub-tile, else at this one.
                 if (u != (first << lm)) __syncthreads();
-                copy_params<SET, C>(B.k, s_k);
+                copy_params<SET>(B.k, s_k);
                 // per-plane pull bases (interior offset folded in) and store bases
                 const int cur = B.phase ^ parity;
                 if (threadIdx.x < V) {
@@ -166,10 +144,10 @@ k_engine_step(const EngineSolve<C>* __restrict__ solves, const EngineTile* __res
             const bool rows = !fast && ya >= k.maxey && yb < k.Ny - k.maxey;
             C f[V];
             if (fast) {
-                take<SET, S, C>(f, [&](auto a) { return sp[a] + cell; });
+                take<SET, S, C, true>(f, [&](auto a) { return sp[a] + cell; });
             } else if (rows || (cell / k.Nx >= k.maxey && cell / k.Nx < k.Ny - k.maxey)) {
                 // nodes away from the walls (the whole sub-tile, or this node of a wall tile)
-                pull_rows_any<SET, S, C>(k, sp, cell, f);
+                pull_rows_any<SET, S, C, true>(k, sp, cell, f);
             } else {
                 const int y = cell / k.Nx;
                 const int x = cell - y * k.Nx;
@@ -267,8 +245,8 @@ __device__ __forceinline__ int xwrap(int x, int Nx) {
 // same terms, in the same order, as wall_dpsi.  In a B step the leaving
 // population b of node m = (x - e_x, j) sits at (m, bbar); in an A step it
 // sits in the ghost row at (m + e_b, b).
-template <class SET, typename S, typename C, bool BOTTOM, bool STEP_A>
-__device__ __forceinline__ double res_wall_dpsi(const KParams<C>& k, const S* sb, int PS, int x) {
+template <class SET, typename S, typename C, bool BOTTOM, bool STEP_A, int MV>
+__device__ __forceinline__ double res_wall_dpsi(const KParams<C, MV>& k, const S* sb, int PS, int x) {
     constexpr int V = SET::R + 2 * SET::P, G = set_maxey<SET>();
     const int Nx = k.Nx;
     auto term = [&](auto bc, int j) {
@@ -288,8 +266,8 @@ __device__ __forceinline__ double res_wall_dpsi(const KParams<C>& k, const S* sb
 }
 
 // Population A of a wall node from shared memory (fill or in-domain value).
-template <class SET, typename S, typename C, bool STEP_A, int A>
-__device__ __forceinline__ C res_wall_value(const KParams<C>& k, const S* sb, int PS, int x, int y,
+template <class SET, typename S, typename C, bool STEP_A, int A, int MV>
+__device__ __forceinline__ C res_wall_value(const KParams<C, MV>& k, const S* sb, int PS, int x, int y,
                                             C pb, C pt) {
     constexpr int G = set_maxey<SET>();
     constexpr int EY = plane_ey<SET>(A);
@@ -303,8 +281,8 @@ __device__ __forceinline__ C res_wall_value(const KParams<C>& k, const S* sb, in
     return ld_val<S, C>(sb[plane_opp<SET>(A) * PS + (ys + G) * Nx + xs]);
 }
 
-template <class SET, typename S, typename C, bool STEP_A, int... I>
-__device__ __forceinline__ void res_pull_wall(const KParams<C>& k, const S* sb, int PS, int x, int y,
+template <class SET, typename S, typename C, bool STEP_A, int MV, int... I>
+__device__ __forceinline__ void res_pull_wall(const KParams<C, MV>& k, const S* sb, int PS, int x, int y,
                                               C* f, std::integer_sequence<int, I...>) {
     constexpr int G = set_maxey<SET>();
     const C pb = y < G ? C(res_wall_dpsi<SET, S, C, true, STEP_A>(k, sb, PS, x)) : C(0);
@@ -312,43 +290,41 @@ __device__ __forceinline__ void res_pull_wall(const KParams<C>& k, const S* sb, 
     ((f[I] = res_wall_value<SET, S, C, STEP_A, I>(k, sb, PS, x, y, pb, pt)), ...);
 }
 
-// Element, relative to the channel's planes, that a node reads population A
-// from (res_src) and writes it to (res_dst).  The slot a population is written
-// to is the slot its opposite was read from.
-template <class SET, int MODE, bool STEP_A, int A>
-__device__ __forceinline__ int res_src(int PS, int Nx, int x, int y) {
+template <class SET, typename S, typename C, int MODE, bool STEP_A, int MV, int... I>
+__device__ __forceinline__ void res_pull(const KParams<C, MV>& k, const S* sb, int PS, int x, int y,
+                                         C* f, std::integer_sequence<int, I...>) {
     constexpr int G = set_maxey<SET>();
-    if constexpr (STEP_A) return A * PS + (y + G) * Nx + x;
-    else return plane_opp<SET>(A) * PS + (y - plane_ey<SET>(A) + G) * Nx + xwrap<-plane_ex<SET>(A), MODE>(x, Nx);
-}
-template <class SET, int MODE, bool STEP_A, int A>
-__device__ __forceinline__ int res_dst(int PS, int Nx, int x, int y) {
-    constexpr int G = set_maxey<SET>();
-    if constexpr (STEP_A) return plane_opp<SET>(A) * PS + (y + G) * Nx + x;
-    else return A * PS + (y + plane_ey<SET>(A) + G) * Nx + xwrap<plane_ex<SET>(A), MODE>(x, Nx);
-}
-
-// Pull (away from the walls), collision and push of one node, its x wrap mode
-// known.
-template <class SET, int N, typename S, typename C, int MODE, bool STEP_A>
-__device__ __forceinline__ CellCoef<C> res_update(const KParams<C>& k, S* sb, int PS, int x, int y, bool wall,
-                                                  unsigned rs, bool want, C* f) {
-    constexpr int V = SET::R + 2 * SET::P;
     const int Nx = k.Nx;
-    if (!wall)
-        for_planes([&](auto a) {
-            f[a] = ld_val<S, C>(sb[res_src<SET, MODE, STEP_A, decltype(a)::value>(PS, Nx, x, y)]);
-        }, std::make_integer_sequence<int, V>{});
-    return finish_node<SET, N, S, C>(k, f, want, rs, [&](auto a, S v) {
-        sb[res_dst<SET, MODE, STEP_A, decltype(a)::value>(PS, Nx, x, y)] = v;
-    });
+    if constexpr (STEP_A) {
+        const int o = (y + G) * Nx + x;
+        ((f[I] = ld_val<S, C>(sb[I * PS + o])), ...);
+    } else {
+        ((f[I] = ld_val<S, C>(sb[plane_opp<SET>(I) * PS + (y - plane_ey<SET>(I) + G) * Nx +
+                                 xwrap<-plane_ex<SET>(I), MODE>(x, Nx)])), ...);
+    }
 }
 
-// The same for an fp64 node, which reads its populations where they lie: a wall
+template <class SET, typename S, typename C, int MODE, bool STEP_A, int MV, int... I>
+__device__ __forceinline__ void res_push(const KParams<C, MV>& k, S* sb, int PS, int x, int y, const C* f,
+                                         unsigned rs, std::integer_sequence<int, I...>) {
+    constexpr int G = set_maxey<SET>();
+    const int Nx = k.Nx;
+    S out[sizeof...(I)];
+    pack_ct<SET, S, C>(f, rs, out);
+    if constexpr (STEP_A) {
+        const int o = (y + G) * Nx + x;
+        ((sb[plane_opp<SET>(I) * PS + o] = out[I]), ...);
+    } else {
+        ((sb[I * PS + (y + plane_ey<SET>(I) + G) * Nx + xwrap<plane_ex<SET>(I), MODE>(x, Nx)] =
+              out[I]), ...);
+    }
+}
+
+// Update of an fp64 node, which reads its populations where they lie: a wall
 // node first writes its wall fills into the slots they would have come from,
 // which only this node touches in this step.
-template <class SET, int N, int MODE, bool STEP_A>
-__device__ __forceinline__ CellCoef<double> res_update64(const KParams<double>& k, double* sb, int PS, int x,
+template <class SET, int N, int MODE, bool STEP_A, int MV>
+__device__ __forceinline__ CellCoef<double> res_update64(const KParams<double, MV>& k, double* sb, int PS, int x,
                                                          int y, bool want) {
     constexpr int G = set_maxey<SET>();
     const int Nx = MODE == 0 ? 1 : k.Nx, o = (y + G) * Nx + x;
@@ -413,16 +389,21 @@ __device__ __forceinline__ void res_node(const EngineSolve<C>& B, S* sb, int PS,
         else if (Nx >= k.maxex) q = res_update64<SET, N, 1, STEP_A>(k, sb, PS, x, y, emit != 0);
         else q = res_update64<SET, N, 2, STEP_A>(k, sb, PS, x, y, emit != 0);
     } else {
+        constexpr auto planes = std::make_integer_sequence<int, V>{};
         C f[V];
-        const bool wall = y < G || y >= Ny - G;
-        if (wall) res_pull_wall<SET, S, C, STEP_A>(k, sb, PS, x, y, f, std::make_integer_sequence<int, V>{});
+        const int mode = Nx == 1 ? 0 : (Nx >= k.maxex ? 1 : 2);
+        if (y >= G && y < Ny - G) {
+            if (mode == 0) res_pull<SET, S, C, 0, STEP_A>(k, sb, PS, x, y, f, planes);
+            else if (mode == 1) res_pull<SET, S, C, 1, STEP_A>(k, sb, PS, x, y, f, planes);
+            else res_pull<SET, S, C, 2, STEP_A>(k, sb, PS, x, y, f, planes);
+        } else {
+            res_pull_wall<SET, S, C, STEP_A>(k, sb, PS, x, y, f, planes);
+        }
+        q = relax_node<SET, N, S, C>(k, f);
         const unsigned rs = sr_seed<S, C>(seed + unsigned(slot) * 0x632be5abu, cell);
-        if (Nx == 1)
-            q = res_update<SET, N, S, C, 0, STEP_A>(k, sb, PS, x, y, wall, rs, emit != 0, f);
-        else if (Nx >= k.maxex)
-            q = res_update<SET, N, S, C, 1, STEP_A>(k, sb, PS, x, y, wall, rs, emit != 0, f);
-        else
-            q = res_update<SET, N, S, C, 2, STEP_A>(k, sb, PS, x, y, wall, rs, emit != 0, f);
+        if (mode == 0) res_push<SET, S, C, 0, STEP_A>(k, sb, PS, x, y, f, rs, planes);
+        else if (mode == 1) res_push<SET, S, C, 1, STEP_A>(k, sb, PS, x, y, f, rs, planes);
+        else res_push<SET, S, C, 2, STEP_A>(k, sb, PS, x, y, f, rs, planes);
     }
     res_emit<C>(B, q, cell, emit);
 }

@@ -28,6 +28,9 @@ struct EngineLaunch {
 template <class SET, int N, typename S>
 cudaError_t engine_step_one(const EngineLaunch& L, cudaStream_t st) {
     using C = CompOf<S>;
+    // not chained like the single-solve steps: persistent blocks fill the GPU and
+    // the groups' launches overlap, early blocks of the next step take slots from
+    // the other group (config of 256 channels: 2 % slower)
     k_engine_step<SET, N, S, C><<<L.grid, kBlock, step_smem<SET, C>(), st>>>(
         static_cast<const EngineSolve<C>*>(L.solves), L.tiles, L.ntiles, L.tile_off, L.counter, L.seed,
         L.parity, L.emit, L.chunk, L.lm);

@@ -74,7 +74,7 @@ struct Source {
 // shuffles form (a0 + a1) + (a2 + a3) -- the bits of wall_dpsi.
 template <int LP, int N, typename S, typename C>
 __global__ void __launch_bounds__(kClusterThreads)
-k_chunk_cluster(const __grid_constant__ KParams<C> k, const S* fin, S* fout, const DevBufs b,
+k_chunk_cluster(const __grid_constant__ KParams<C, 2 * LP + 1> k, const S* fin, S* fout, const DevBufs b,
                 int K, int rows, int emit_prev, int nb, int nt) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int G = 32 / LP;
@@ -295,9 +295,13 @@ cudaError_t launch_chunk_cluster_t(const KParams<C>& k, const ClusterPlan& pl, c
     const C* src = static_cast<const C*>(fin);
     C* dst = static_cast<C*>(fout);
     int rows = pl.rows, ep = emit_prev ? 1 : 0, nb = pl.nb, nt = pl.nt;
-    void* args[] = {const_cast<KParams<C>*>(&k), &src, &dst, const_cast<DevBufs*>(&b),
-                    &K, &rows, &ep, &nb, &nt};
-    return cudaLaunchKernelExC(&cfg, fn, args);
+    auto launch = [&](auto ks) {
+        void* args[] = {&ks, &src, &dst, const_cast<DevBufs*>(&b), &K, &rows, &ep, &nb, &nt};
+        return cudaLaunchKernelExC(&cfg, fn, args);
+    };
+    if (pl.LP == 8) return launch(shrink_params<17>(k));
+    if (pl.LP == 16) return launch(shrink_params<33>(k));
+    return launch(shrink_params<65>(k));
 }
 
 int plan_cluster(const KParams<double>& k, int N, int LP, ClusterPlan& pl) {

@@ -3,7 +3,10 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <stddef.h>
 #include <stdint.h>
+
+#include <cstring>
 
 #include <vector>
 
@@ -36,9 +39,14 @@ template <> struct FxOf<double> { using type = fx::Consts; };
 // Per-solve constants, passed by value to every kernel (__grid_constant__).
 // Planes are in the solver's internal order: R rest planes (R = 0 or 1),
 // then the P "positive" members of the +-e pairs, then their P negatives in
-// the same order, so plane R + P + p holds -e of plane R + p.
-template <typename C>
+// the same order, so plane R + P + p holds -e of plane R + p.  The arrays hold MV
+// planes: the solver's record has room for any set, a kernel of a known set
+// takes one of its own size (shrink_params), because the host copies a launch's
+// parameters: with the 10 KB (fp32) and 17 KB (fp64) records a launch took 6
+// and 17 us, more than a small channel's step.
+template <typename C, int MV = LBM_MAX_V>
 struct KParams {
+    static constexpr int MP = MV / 2;
     int Nx, Ny, ncell;           // ncell = Nx * Ny
     int R, P, V;
     int maxey;                   // max |e_y|: rows within maxey of a wall
@@ -49,33 +57,33 @@ struct KParams {
     int emit;                    // 1: write fp64 rho, u of this step; 2: add them
     unsigned int seed;           // step counter: stochastic rounding of 16-bit stores
     long long plane;             // elements per plane = ncell
-    int ex[LBM_MAX_V], ey[LBM_MAX_V];
-    int sx[LBM_MAX_V];           // e_x mod Nx, in [0, Nx)
-    int off[LBM_MAX_V];          // e_y Nx + e_x: pull offset of an interior node
-    int dx[LBM_MAX_V];           // e_x - sx: offset correction when x - e_x wraps
+    int ex[MV], ey[MV];
+    int sx[MV];           // e_x mod Nx, in [0, Nx)
+    int off[MV];          // e_y Nx + e_x: pull offset of an interior node
+    int dx[MV];           // e_x - sx: offset correction when x - e_x wraps
     // per launch: plane base pointers of the source lattice shifted by the
     // interior pull offset (srcf[a] = src + a plane - off[a]) and of the
     // destination lattice (dstp[a] = dst + a plane)
-    const void* srcf[LBM_MAX_V];
-    void* dstp[LBM_MAX_V];
-    double w[LBM_MAX_V];         // weights (fp64) for the initial state
-    C cw[LBM_MAX_V];             // weights in the compute type, for the wall fill
+    const void* srcf[MV];
+    void* dstp[MV];
+    double w[MV];         // weights (fp64) for the initial state
+    C cw[MV];             // weights in the compute type, for the wall fill
     // 16-bit storage only: stored h_a = d_a / (w_a S), S a per-solve power of 2
-    C sw[LBM_MAX_V];             // w_a S      (load:  d = h * sw)
-    C isw[LBM_MAX_V];            // 1/(w_a S)  (store: h = d * isw)
+    C sw[MV];             // w_a S      (load:  d = h * sw)
+    C isw[MV];            // 1/(w_a S)  (store: h = d * isw)
     // 16-bit storage, compiled velocity sets: the kernels keep h itself in
     // registers; the moment sums of d = w S h weigh h with these (pair p):
-    C hw[kMaxPairs], hwx[kMaxPairs], hwy[kMaxPairs];        // w S, w S e_x, w S e_y
-    C hwxx[kMaxPairs], hwxy[kMaxPairs], hwyy[kMaxPairs];    // w S e_x^2, w S e_x e_y, w S e_y^2
+    C hw[MP], hwx[MP], hwy[MP];        // w S, w S e_x, w S e_y
+    C hwxx[MP], hwxy[MP], hwyy[MP];    // w S e_x^2, w S e_x e_y, w S e_y^2
     C hw_rest;                   // w_rest S
     C fill_h;                    // 1/S: the wall fill dPsi w_a in units of w_a S
     C om_s;                      // omega / S: relaxation target in units of w_a S
     double inv_den;              // 1 / sum_{e_y > 0} e_y w  (= same for e_y < 0)
     // per pair p, positive member e = (ex, ey):
-    C pex[kMaxPairs], pey[kMaxPairs];
-    C pexx[kMaxPairs], pexy2[kMaxPairs], peyy[kMaxPairs];   // ex^2, 2 ex ey, ey^2
-    C pge[kMaxPairs];            // c g.e
-    C pomw[kMaxPairs];           // omega w_p
+    C pex[MP], pey[MP];
+    C pexx[MP], pexy2[MP], peyy[MP];   // ex^2, 2 ex ey, ey^2
+    C pge[MP];            // c g.e
+    C pomw[MP];           // omega w_p
     C omw_rest;                  // omega w_rest
     // scalars
     C c, c2, tau, dt, hdt, omega, one_m_omega, gx, gy;
@@ -85,6 +93,64 @@ struct KParams {
     C hdt_gx, hdt_gy, tgx, tgy, ttc2, htc2, tc, cg;
     typename FxOf<C>::type fx;
 };
+
+// The parts of src that a set of at most MV planes uses, to a record with room
+// for MD >= MV: cp(dst, src, 4-byte words) for each contiguous run.
+template <int MV, typename C, int MD, class CP>
+#if defined(__CUDACC__)
+__host__ __device__ __forceinline__
+#else
+inline
+#endif
+void copy_params_by(const KParams<C>& src, KParams<C, MD>& dst, const CP& cp) {
+    constexpr int MP = MV / 2, cw = int(sizeof(C) / 4);
+    static_assert(offsetof(KParams<C>, seed) == 12 * 4 && offsetof(KParams<C>, om_s) == offsetof(KParams<C>, hw_rest) + 2 * sizeof(C),
+                  "runs below");
+    auto run = [&](auto* d, const auto* s, int words) {
+        cp(reinterpret_cast<int*>(d), reinterpret_cast<const int*>(s), words);
+    };
+    run(&dst.Nx, &src.Nx, 13);                             // Nx .. seed
+    run(&dst.plane, &src.plane, 2);
+    run(dst.ex, src.ex, MV);
+    run(dst.ey, src.ey, MV);
+    run(dst.sx, src.sx, MV);
+    run(dst.off, src.off, MV);
+    run(dst.dx, src.dx, MV);
+    run(dst.srcf, src.srcf, 2 * MV);
+    run(dst.dstp, src.dstp, 2 * MV);
+    run(dst.w, src.w, 2 * MV);
+    run(dst.cw, src.cw, cw * MV);
+    run(dst.sw, src.sw, cw * MV);
+    run(dst.isw, src.isw, cw * MV);
+    run(dst.hw, src.hw, cw * MP);
+    run(dst.hwx, src.hwx, cw * MP);
+    run(dst.hwy, src.hwy, cw * MP);
+    run(dst.hwxx, src.hwxx, cw * MP);
+    run(dst.hwxy, src.hwxy, cw * MP);
+    run(dst.hwyy, src.hwyy, cw * MP);
+    // runs of members of one type only: the padding between members of
+    // different alignment depends on MV
+    run(&dst.hw_rest, &src.hw_rest, 3 * cw);               // hw_rest, fill_h, om_s
+    run(&dst.inv_den, &src.inv_den, 2);
+    run(dst.pex, src.pex, cw * MP);
+    run(dst.pey, src.pey, cw * MP);
+    run(dst.pexx, src.pexx, cw * MP);
+    run(dst.pexy2, src.pexy2, cw * MP);
+    run(dst.peyy, src.peyy, cw * MP);
+    run(dst.pge, src.pge, cw * MP);
+    run(dst.pomw, src.pomw, cw * MP);
+    run(&dst.omw_rest, &src.omw_rest,
+        int((offsetof(KParams<C>, cg) - offsetof(KParams<C>, omw_rest)) / 4) + cw);
+    if constexpr (sizeof(C) == 8) run(&dst.fx, &src.fx, int(sizeof(src.fx) / 4));
+}
+
+// A record of MV planes for a launch.
+template <int MV, typename C>
+inline KParams<C, MV> shrink_params(const KParams<C>& k) {
+    KParams<C, MV> d;
+    copy_params_by<MV>(k, d, [](int* t, const int* s, int words) { std::memcpy(t, s, size_t(words) * 4); });
+    return d;
+}
 
 // Device buffers of one solver.
 struct DevBufs {
