@@ -94,8 +94,11 @@ struct Consts {
     // rows [0, nx): e = (ax, 0); [nx, ny): (0, ay); [ny, nd): four velocities
     int nx, ny, nd, rest;    // rest: 1 if plane 0 is the rest population
     Mul om0;                 // omega w of the rest population = om0 2^-oe0
-    int oe0, pad;
+    int oe0, fam;            // fam: see FamilyFormat, -1: none fits
     Row row[kMaxRows];
+    // per pair (plane order): omega w = pom 2^-poe
+    Mul pom[kMaxRows];
+    int poe[kMaxRows];
 };
 
 LBM_HD i64 mulw(int a, int b) { return i64(a) * b; }
@@ -242,6 +245,21 @@ LBM_CX int c2_point(int emax) { return emax > 4 ? 63 : 61; }
 LBM_CX int extra2(int emax) { return emax > 4 ? 2 : 0; }
 LBM_CX int extra3(int emax) { return emax > 4 ? 5 : 0; }
 
+// The binary points of a set's fixed-point form.
+template <class SET>
+struct Format {
+    static constexpr int EMAX = set_emax<SET>(), S0 = guard_bits<SET>(), KS = kshift<SET>();
+    static constexpr int S2 = extra2(EMAX), S3 = extra3(EMAX), C2 = c2_point(EMAX);
+};
+// The same for a kernel that knows only the number LP of lanes per node (pairs
+// at most LP) and, for LP = 16, which of the two: 0 for components up to 4, 1 for
+// up to 8, 2 above.  SetInfo::fam says which one fits a set.
+template <int FAM>
+struct FamilyFormat {
+    static constexpr int EMAX = FAM == 0 ? 4 : (FAM == 1 ? 8 : 16), S0 = FAM == 2 ? 5 : 4, KS = ilog2_up(EMAX);
+    static constexpr int S2 = extra2(EMAX), S3 = extra3(EMAX), C2 = c2_point(EMAX);
+};
+
 struct Sums {
     i64 d, jx, jy, kxx, kxy, kyy;
 };
@@ -306,10 +324,10 @@ LBM_HD i64 const_q(i64 mant, int exp, int q, unsigned& frac) {
 // are multiples of 2^-62.  M = rho X, H = rho X X / 2, t = rho X X X / 2,
 // a = rho X^4 / 4 (and the mixed products).  Shifts left before a product use
 // the room the bounds leave, so that a product loses less than a unit.
-template <class SET, int N, bool FORCE>
+template <class FMT, int N, bool FORCE>
 LBM_HD bool coefs(const Consts& k, const Sums& m, int E, Poly& p) {
-    constexpr int EMAX = set_emax<SET>(), S2 = extra2(EMAX), S3 = extra3(EMAX), C2 = c2_point(EMAX);
-    const int q = 1074 + guard_bits<SET>() - E;
+    constexpr int S2 = FMT::S2, S3 = FMT::S3, C2 = FMT::C2;
+    const int q = 1074 + FMT::S0 - E;
     const float fd = hif(m.d), fj = fabsf_(hif(m.jx)) + fabsf_(hif(m.jy));
     float fk = 0.f;
     if (FORCE && N >= 3) fk = fabsf_(hif(m.kxx)) + fabsf_(hif(m.kxy)) + fabsf_(hif(m.kyy));
@@ -532,7 +550,7 @@ LBM_HD bool collide(const Consts& k, double omo, Sums& m, int& E, const GET& get
         }
     });
     Poly p;
-    if (!coefs<SET, N, FORCE>(k, m, E, p)) return false;
+    if (!coefs<Format<SET>, N, FORCE>(k, m, E, p)) return false;
     phase();
     // G = Ge +- Go of e and -e: Ge = Ee + sx sy Eo, Go = sx Ox + sy Oy with sx, sy
     // the signs of the components (see PolyCoef); T = G omega w
@@ -585,12 +603,35 @@ LBM_HD bool collide(const Consts& k, double omo, Sums& m, int& E, const GET& get
     return true;
 }
 
+// Target of the pair of velocity (ex, ey), before the weight: Ge +- Go for the
+// member and its negative (the polynomial in e evaluated for one pair).
+template <class FMT, int N>
+LBM_HD void pair_target(const Poly& p, int ex, int ey, i64& Ge, i64& Go) {
+    const int x2 = ex * ex, y2 = ey * ey, xy = ex * ey;
+    i64 ev = madk(madk(0, x2, p.c20), y2, p.c02) + i64(xy) * p.c11, od = 0;
+    if (N >= 4) {
+        ev = madk(madk(madk(ev, x2 * x2, p.c40), xy * xy, p.c22), y2 * y2, p.c04);
+        ev += i64(xy * x2) * p.c31 + i64(xy * y2) * p.c13;
+    }
+    if (N >= 3)
+        od = i64(x2 * ex) * p.d30 + i64(xy * ey) * p.d12 + i64(y2 * ey) * p.d03 + i64(xy * ex) * p.d21;
+    Ge = p.c00 + sh_(ev, -FMT::S2);
+    Go = i64(ex) * p.d10 + i64(ey) * p.d01 + sh_(od, -FMT::S3);
+}
+
 // What the constants need to know of a velocity set.
 struct SetInfo {
-    int emax, ks, s0;
+    int emax, ks, s0, fam;
 };
 template <class SET>
-LBM_CX SetInfo set_info() { return SetInfo{set_emax<SET>(), kshift<SET>(), guard_bits<SET>()}; }
+LBM_CX SetInfo set_info() {
+    using F = Format<SET>;
+    const int fam = F::EMAX <= 4 ? 0 : (F::EMAX <= 8 ? 1 : 2);
+    const bool fits = fam == 0 ? F::S0 == FamilyFormat<0>::S0 && F::KS == FamilyFormat<0>::KS
+                     : fam == 1 ? F::S0 == FamilyFormat<1>::S0 && F::KS == FamilyFormat<1>::KS
+                                : F::S0 == FamilyFormat<2>::S0 && F::KS == FamilyFormat<2>::KS;
+    return SetInfo{F::EMAX, F::KS, F::S0, fits ? fam : -1};
+}
 
 // Host: the constants of a solve (lattice speed c, relaxation time tau, time
 // step dt, force g along x) of a set with planes e = (ex, ey), weights w, the
@@ -662,6 +703,9 @@ inline Consts make_consts(double c_, double tau_, double dt_, double g_, int R, 
     k.ga = f3 * (4.0f + 4.0f * k.c2f * em * em) * em;
     const double omega = dt_ / (tau_ + 0.5 * dt_);
     k.rest = R;
+    k.fam = si.fam;
+    if (P > kMaxRows) k.ok = 0;
+    for (int p = 0; p < P && k.ok; ++p) k.pom[p] = to_weight(omega * w[R + p], k.poe[p], k.ok);
     if (R) k.om0 = to_weight(omega * w[0], k.oe0, k.ok);
     for (int kind = 0; kind < 3; ++kind) {
         for (int p = 0; p < P && k.ok; ++p) {

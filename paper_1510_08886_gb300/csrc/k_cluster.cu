@@ -72,8 +72,8 @@ struct Source {
 // The wall sums are split over the first four lanes of a wall node: lane j adds
 // the terms j, j + 4, ... in order, exactly accumulator j of Acc4, and two
 // shuffles form (a0 + a1) + (a2 + a3) -- the bits of wall_dpsi.
-template <int LP, int N, typename S, typename C>
-__global__ void __launch_bounds__(kClusterThreads)
+template <int LP, int N, int MAXT, typename S, typename C>
+__global__ void __launch_bounds__(MAXT)
 k_chunk_cluster(const __grid_constant__ KParams<C, 2 * LP + 1> k, const S* fin, S* fout, const DevBufs b,
                 int K, int rows, int emit_prev, int nb, int nt) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -121,6 +121,7 @@ k_chunk_cluster(const __grid_constant__ KParams<C, 2 * LP + 1> k, const S* fin, 
     const bool act = node && p < k.P;
     const bool has0 = node && p == 0 && k.R;
     const PairConst<C> pc = pair_const(k, act ? p : 0);
+    const PairFx pf = pair_fx(k, act ? p : 0);
     auto source = [&](int a) -> Source<S, C> {
         Source<S, C> src{nullptr, 0, k.cw[a]};
         const int ys = y - k.ey[a];
@@ -167,7 +168,7 @@ k_chunk_cluster(const __grid_constant__ KParams<C, 2 * LP + 1> k, const S* fin, 
         const C fm = act ? value(sm, pb, pt, to, k.R + k.P + p) : C(0);
         const C f0 = has0 ? value(s0, pb, pt, to, 0) : C(0);
         auto put = [&](int a, C v) { dst[a * lplane + cl] = S(v); };
-        const CellCoef<C> q = warp_node<LP, N, C>(k, p, node, pc, fp, fm, f0, put);
+        const CellCoef<C> q = warp_node_any<LP, N, C>(k, p, node, pc, pf, fp, fm, f0, s >= K - 2, put);
         if (node && p == 0) {
             if (s == K - 1) store_moments<C>(q, int(g0 + cl), b);
             else if (emit_prev && s == K - 2) b.prev_ux[g0 + cl] = (double)q.ux;
@@ -182,25 +183,32 @@ k_chunk_cluster(const __grid_constant__ KParams<C, 2 * LP + 1> k, const S* fin, 
     }
 }
 
-template <int LP, int N, typename C>
+template <int LP, int N, int MAXT, typename C>
 void* cluster_kernel() {
-    return reinterpret_cast<void*>(&k_chunk_cluster<LP, N, C, C>);
+    return reinterpret_cast<void*>(&k_chunk_cluster<LP, N, MAXT, C, C>);
 }
 
-template <typename C>
-void* pick_kernel(int N, int LP) {
+template <int MAXT, typename C>
+void* pick_sized(int N, int LP) {
     switch (LP * 10 + N) {
-        case 82: return cluster_kernel<8, 2, C>();
-        case 83: return cluster_kernel<8, 3, C>();
-        case 84: return cluster_kernel<8, 4, C>();
-        case 162: return cluster_kernel<16, 2, C>();
-        case 163: return cluster_kernel<16, 3, C>();
-        case 164: return cluster_kernel<16, 4, C>();
-        case 322: return cluster_kernel<32, 2, C>();
-        case 323: return cluster_kernel<32, 3, C>();
-        case 324: return cluster_kernel<32, 4, C>();
+        case 82: return cluster_kernel<8, 2, MAXT, C>();
+        case 83: return cluster_kernel<8, 3, MAXT, C>();
+        case 84: return cluster_kernel<8, 4, MAXT, C>();
+        case 162: return cluster_kernel<16, 2, MAXT, C>();
+        case 163: return cluster_kernel<16, 3, MAXT, C>();
+        case 164: return cluster_kernel<16, 4, MAXT, C>();
+        case 322: return cluster_kernel<32, 2, MAXT, C>();
+        case 323: return cluster_kernel<32, 3, MAXT, C>();
+        case 324: return cluster_kernel<32, 4, MAXT, C>();
         default: return nullptr;
     }
+}
+
+// fp64 in 256-thread blocks may use all the registers it wants; more rows per CTA
+// than that need the larger block's 80.
+template <typename C>
+void* pick_kernel(int N, int LP, int threads) {
+    return sizeof(C) == 8 && threads <= 256 ? pick_sized<256, C>(N, LP) : pick_sized<kClusterThreads, C>(N, LP);
 }
 
 cudaLaunchConfig_t cluster_config(const ClusterPlan& pl, cudaStream_t st, cudaLaunchAttribute* at) {
@@ -228,8 +236,6 @@ cudaLaunchConfig_t cluster_config(const ClusterPlan& pl, cudaStream_t st, cudaLa
 template <typename C>
 int plan_cluster_t(const KParams<C>& k, int N, int LP, ClusterPlan& pl) {
     pl = ClusterPlan{};
-    void* fn = pick_kernel<C>(N, LP);
-    if (!fn) return 0;
     int dev = 0, optin = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
@@ -247,6 +253,8 @@ int plan_cluster_t(const KParams<C>& k, int N, int LP, ClusterPlan& pl) {
         const int ctas = (k.Ny + rows - 1) / rows;
         const int groups = (rows * k.Nx + G - 1) / G;      // warps of work per CTA
         if (groups > kClusterThreads / 32) continue;
+        void* fn = pick_kernel<C>(N, LP, 32 * groups);
+        if (!fn) return 0;
         const size_t need = ((size_t(2) * k.V * rows * k.Nx * sizeof(C) + 15) & ~size_t(15)) +
                             size_t(nb + nt) * sizeof(WallTerm<C>);
         const size_t smem = std::max(need, size_t(kClusterSmemPad));
@@ -288,7 +296,7 @@ template <typename C>
 cudaError_t launch_chunk_cluster_t(const KParams<C>& k, const ClusterPlan& pl, const void* fin,
                                    void* fout, const DevBufs& b, int K, bool emit_prev,
                                    cudaStream_t st) {
-    void* fn = pick_kernel<C>(pl.N, pl.LP);
+    void* fn = pick_kernel<C>(pl.N, pl.LP, pl.threads);
     if (!fn || pl.ctas < 1 || K < 1) return cudaErrorInvalidValue;
     cudaLaunchAttribute at[1];
     const cudaLaunchConfig_t cfg = cluster_config(pl, st, at);

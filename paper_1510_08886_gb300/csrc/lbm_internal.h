@@ -199,7 +199,7 @@ inline int warp_path_lanes(int P, long long ncell) {
 // Resident chunks of a tiny fp64 or fp32 channel on one thread-block cluster
 // (k_cluster.cu): CTAs of at most kClusterThreads threads, shared memory padded
 // to kClusterSmemPad (more than half an SM's) so that no two share an SM.
-constexpr int kClusterThreads = 256;
+constexpr int kClusterThreads = 768;
 constexpr int kClusterSmemPad = 116 * 1024;
 constexpr long kClusterMaxK = 4096;           // steps per launch in lbm_step
 struct ClusterPlan {

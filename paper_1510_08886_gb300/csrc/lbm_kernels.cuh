@@ -868,6 +868,19 @@ __device__ __forceinline__ void for_planes(const FN& fn, std::integer_sequence<i
     (fn(Plane<I>{}), ...);
 }
 
+// rho and u (Eq. nm.10) from the sums of a node, value m.d 2^(E - 1075 - S0).
+template <int S0, int MV>
+__device__ __forceinline__ void fx_moments(const KParams<double, MV>& k, const fx::Sums& m, int E,
+                                           CellCoef<double>& q) {
+    const double u = __hiloint2double((E + 1 - S0) << 20, 0);      // two exact steps
+    auto val = [&](long long v) { return mul_rn(mul_rn(double(v), 0x1p-53), u); };
+    q.drho = val(m.d);
+    q.rho = 1.0 + q.drho;
+    const double inv = 1.0 / q.rho;
+    q.ux = fma(mul_rn(k.c, val(m.jx)), inv, k.hdt_gx);
+    q.uy = fma(mul_rn(k.c, val(m.jy)), inv, k.hdt_gy);
+}
+
 // fp64 collision of a node of a compiled set (get, put: see fx::collide).  The
 // moments rho, u of the result are valid when want is set; drho and rho are
 // always fit for flag_density.
@@ -882,16 +895,7 @@ __device__ __forceinline__ CellCoef<double> collide64(const KParams<double, MV>&
     CellCoef<double> q;
     q.drho = 0.0;
     q.rho = 1.0;
-    if (want) {
-        // sums times 2^(E - 1075 - S0), in two exact steps
-        const double u = __hiloint2double((E + 1 - fx::guard_bits<SET>()) << 20, 0);
-        auto val = [&](long long v) { return mul_rn(mul_rn(double(v), 0x1p-53), u); };
-        q.drho = val(m.d);
-        q.rho = 1.0 + q.drho;
-        const double inv = 1.0 / q.rho;
-        q.ux = fma(mul_rn(k.c, val(m.jx)), inv, k.hdt_gx);
-        q.uy = fma(mul_rn(k.c, val(m.jy)), inv, k.hdt_gy);
-    }
+    if (want) fx_moments<fx::guard_bits<SET>()>(k, m, E, q);
     return q;
 }
 
@@ -1284,6 +1288,107 @@ __device__ __forceinline__ CellCoef<C> warp_node(const KParams<C, MV>& k, int p,
     return q;
 }
 
+// Fixed-point constants of a lane's pair (fx64.cuh).
+struct PairFx {
+    fx::Mul om;
+    int oe, lg, ex, ey;
+};
+template <typename C, int MV>
+__device__ __forceinline__ PairFx pair_fx(const KParams<C, MV>& k, int p) {
+    PairFx f{};
+    if constexpr (sizeof(C) == 8) {
+        if (k.fx.ok) {
+            f.ex = k.ex[k.R + p];
+            f.ey = k.ey[k.R + p];
+            const int m = max(max(abs(f.ex), abs(f.ey)), 1);
+            f.lg = 32 - __clz(m - 1);
+            f.om = k.fx.pom[p];
+            f.oe = k.fx.poe[p];
+        }
+    }
+    return f;
+}
+
+// warp_node in fixed point: the same lanes and roles.  ok: the node was in range
+// (the same on all its lanes); nothing is put otherwise.  The coefficients cost
+// ~700 integer instructions on every lane against ~100 FP64 ones of 64 cycles.
+template <int LP, int N, bool FORCE, class FMT, class PUT, int MV>
+__device__ __forceinline__ CellCoef<double> warp_node_fx(const KParams<double, MV>& k, int p, bool node,
+                                                         const PairFx& pc, double fp, double fm, double f0,
+                                                         bool want, bool& ok, const PUT& put) {
+    constexpr unsigned FULL = 0xffffffffu;
+    constexpr int S0 = FMT::S0;
+    const bool act = node && p < k.P;
+    unsigned t = max(unsigned(k.fx.emin) << 20,
+                     max(max(fx::key(fp, pc.lg), fx::key(fm, pc.lg)), fx::key(f0, 0)));
+#pragma unroll
+    for (int o = LP / 2; o > 0; o >>= 1) t = max(t, __shfl_xor_sync(FULL, t, o));
+    const int E = int(t >> 20);
+    CellCoef<double> q{};
+    // (out of range: any E will do, the result is not used)
+    const int Es = min(E, 1021);
+    const long long vp = fx::to_fixed<S0>(fp, Es), vm = fx::to_fixed<S0>(fm, Es);
+    const long long sum = vp + vm, dif = vp - vm;
+    const long long ks = (sum + (1ll << FMT::KS >> 1)) >> FMT::KS;
+    const int ex = act ? pc.ex : 0, ey = act ? pc.ey : 0;
+    long long m[6] = {sum + fx::to_fixed<S0>(f0, Es), ex * dif, ey * dif,
+                      (ex * ex) * ks, (ex * ey) * ks, (ey * ey) * ks};
+    node_sum6<LP, long long>(m, p);
+    const fx::Sums s{m[0], m[1], m[2], m[3], m[4], m[5]};
+    fx::Poly c;
+    ok = E <= 1021 && fx::coefs<FMT, N, FORCE>(k.fx, s, Es, c);
+    if (!ok || !node) return q;
+    const int eb = Es + 10 + 64 - S0;
+    if (act) {
+        long long Ge, Go;
+        fx::pair_target<FMT, N>(c, pc.ex, pc.ey, Ge, Go);
+        Ge = fx::mulc(Ge, pc.om);
+        Go = fx::mulc(Go, pc.om);
+        put(k.R + p, fx::relax(k.one_m_omega, fp, Ge + Go, eb - pc.oe));
+        put(k.R + k.P + p, fx::relax(k.one_m_omega, fm, Ge - Go, eb - pc.oe));
+    }
+    if (p == 0 && k.R) put(0, fx::relax(k.one_m_omega, f0, fx::mulc(c.c00, k.fx.om0), eb - k.fx.oe0));
+    q.drho = 0.0;
+    q.rho = 1.0;
+    if (want) fx_moments<S0>(k, s, Es, q);
+    return q;
+}
+
+// warp_node, in fixed point where it applies.  A node outside its range takes
+// the FP64 form, with the whole warp in step (the forms shuffle).
+template <int LP, int N, typename C, class PUT, int MV>
+__device__ __forceinline__ CellCoef<C> warp_node_any(const KParams<C, MV>& k, int p, bool node,
+                                                     const PairConst<C>& pc, const PairFx& pf, C fp, C fm, C f0,
+                                                     bool want, const PUT& put) {
+    if constexpr (sizeof(C) == 8) {
+        // (the compiled sets of P <= 8, 16 and 32 pairs are of these families)
+        const bool fits = LP == 8 ? k.fx.fam == 0 : (LP == 16 ? k.fx.fam == 0 || k.fx.fam == 2 : k.fx.fam == 1);
+        if (k.fx.ok && fits) {
+            bool ok = false;
+            CellCoef<C> q{};
+            auto go = [&](auto fmt) {
+                using F = decltype(fmt);
+                q = k.force ? warp_node_fx<LP, N, true, F>(k, p, node, pf, fp, fm, f0, want, ok, put)
+                            : warp_node_fx<LP, N, false, F>(k, p, node, pf, fp, fm, f0, want, ok, put);
+            };
+            if constexpr (LP == 8) {
+                go(fx::FamilyFormat<0>{});
+            } else if constexpr (LP == 16) {
+                if (k.fx.fam == 0) go(fx::FamilyFormat<0>{});
+                else go(fx::FamilyFormat<2>{});
+            } else {
+                go(fx::FamilyFormat<1>{});
+            }
+            if (__all_sync(0xffffffffu, ok)) return q;
+            const CellCoef<C> r = warp_node<LP, N, C>(k, p, node, pc, fp, fm, f0, [&](int a, C v) {
+                if (!ok) put(a, v);
+            });
+            return ok ? q : r;
+        }
+    }
+    return warp_node<LP, N, C>(k, p, node, pc, fp, fm, f0, put);
+}
+
 // Step for tiny channels: warp_node on every node, one warp per block, so a
 // channel of a few hundred nodes spreads over many SMs instead of running on
 // one (the fp64 step of a 64-node channel is otherwise bound by a single SM's
@@ -1326,7 +1431,8 @@ k_step_warp(const __grid_constant__ KParams<C, 2 * LP + 1> k, const S* src, S* d
     const C f0 = (node && p == 0 && k.R) ? value(0) : C(0);
     unsigned rs = sr_seed<S, C>(k.seed, cell);
     auto put = [&](int a, C v) { dst[(long long)a * k.plane + cell] = st_pop<S, C>(k, v, a, rs); };
-    const CellCoef<C> q = warp_node<LP, N, C>(k, p, node, pc, fp, fm, f0, put);
+    const CellCoef<C> q = warp_node_any<LP, N, C>(k, p, node, pc, pair_fx(k, act ? p : 0), fp, fm, f0,
+                                                  k.emit != 0, put);
     if (node && p == 0) {
         emit_moments<C>(k, q, cell, b);
         flag_density<C>(q, b.status);

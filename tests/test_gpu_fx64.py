@@ -68,3 +68,12 @@ def test_resident_and_tiled_engine_bitwise(name, N, Nx, Ny):
     assert np.array_equal(out[0][0], out[1][0])
     for a, b in zip(out[0][1], out[1][1]):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("name,N", SETS)
+@pytest.mark.parametrize("Nx,Ny", [(5, 29), (1, 600)])
+@pytest.mark.parametrize("amplitude,mach", [(1e-3, 1e-2), (0.3, 0.1)])
+def test_small_channels_on_lanes(name, N, Nx, Ny, amplitude, mach):
+    """Several lanes per node, resident on a cluster of small or large blocks;
+    the second flow takes the general form on some nodes of a warp."""
+    _compare(name, N, Nx, Ny, 7, amplitude=amplitude, mach=mach)
