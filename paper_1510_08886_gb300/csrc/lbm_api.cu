@@ -34,6 +34,7 @@ struct lbm_solver : lbm::SolveSpec {
     // tiny fp64 / fp32 channels: chunks of steps resident on one thread-block cluster
     lbm::ClusterPlan cl{};
     bool resident = true;
+    std::vector<char> readback;      // lbm_moments of a small channel
 };
 
 namespace lbm {
@@ -46,6 +47,7 @@ using lbm::elem_bytes;
 
 namespace {
 
+constexpr size_t kSmallRead = 128 << 10;
 constexpr unsigned kStateMagic = 0x4c424d31u;   // "LBM1"
 
 struct StateHeader {
@@ -64,6 +66,8 @@ bool is16(int p) { return p == LBM_FP16 || p == LBM_BF16; }
 struct Layout {
     size_t f0, f1, rho, ux, uy, prev, partial, results, status, total;
 };
+
+constexpr size_t kResultsToStatus = 256;    // the status word follows the results
 
 Layout layout(int V, size_t ncell, size_t elem) {
     Layout L{};
@@ -252,11 +256,6 @@ void fill_params_impl(const lbm::SolveSpec* s, KParams<C>& k) {
 int cuda_status(cudaError_t e) {
     if (e == cudaSuccess) return LBM_OK;
     return e == cudaErrorMemoryAllocation ? LBM_ENOMEM : LBM_ECUDA;
-}
-
-__global__ void k_fill(double* p, int n, double v) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) p[i] = v;
 }
 
 // Partial sums for the fp64 reductions: per block, sum of u_x and
@@ -449,17 +448,28 @@ int launch_init(lbm_solver* s, const double* rho_dev) {
     return cuda_status(e);
 }
 
+// The four reduction results and the status word, which follows them in the
+// workspace, in one copy: an error of the copy, else the solve's status.
+int read_results(lbm_solver* s, double out[4]) {
+    unsigned char host[260];
+    static_assert(sizeof(host) == kResultsToStatus + sizeof(unsigned), "layout");
+    cudaError_t e = cudaMemcpyAsync(host, s->b.results, sizeof(host), cudaMemcpyDeviceToHost, s->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+    if (e != cudaSuccess) return cuda_status(e);
+    std::memcpy(out, host, 4 * sizeof(double));
+    unsigned st = 0;
+    std::memcpy(&st, host + kResultsToStatus, sizeof(st));
+    return st ? LBM_ENONFINITE : LBM_OK;
+}
+
 int reduce(lbm_solver* s, bool with_prev, double out[4]) {
     const int n = s->Nx * s->Ny;
     k_reduce_partial<<<lbm::kReduceBlocks, lbm::kReduceThreads, 0, s->stream>>>(
         s->b.ux, with_prev ? s->b.prev_ux : nullptr, n, s->b.partial);
     k_reduce_final<<<1, 256, 0, s->stream>>>(s->b.partial, lbm::kReduceBlocks, s->b.ux, s->Nx,
                                              s->Ny, s->tau, s->g, s->Kn, s->b.results);
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaMemcpyAsync(out, s->b.results, 4 * sizeof(double),
-                                              cudaMemcpyDeviceToHost, s->stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
-    return cuda_status(e);
+    const cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? read_results(s, out) : cuda_status(e);
 }
 
 int read_status(lbm_solver* s) {
@@ -728,14 +738,10 @@ void lbm_destroy(lbm_solver* s) {
 
 int lbm_init(lbm_solver* s, const double* rho_host) {
     if (!s) return LBM_EINVAL;
+    if (!rho_host) return launch_init(s, nullptr);
     const int n = s->Nx * s->Ny;
-    cudaError_t e;
-    if (rho_host)
-        e = cudaMemcpyAsync(s->b.prev_ux, rho_host, size_t(n) * 8, cudaMemcpyHostToDevice, s->stream);
-    else {
-        k_fill<<<(n + 255) / 256, 256, 0, s->stream>>>(s->b.prev_ux, n, 1.0);
-        e = cudaGetLastError();
-    }
+    const cudaError_t e =
+        cudaMemcpyAsync(s->b.prev_ux, rho_host, size_t(n) * 8, cudaMemcpyHostToDevice, s->stream);
     if (e != cudaSuccess) return cuda_status(e);
     return launch_init(s, s->b.prev_ux);
 }
@@ -793,21 +799,11 @@ int lbm_run_to_steady(lbm_solver* s, double tol, long max_steps, long check_ever
     while (s->steps < max_steps) {
         const long n = std::min(check_every, max_steps - s->steps);
         double r[4];
-        if (graphs) {
-            if ((rc = graph_chunk(s, n))) break;
-            cudaError_t e = cudaMemcpyAsync(r, s->b.results, 4 * sizeof(double),
-                                            cudaMemcpyDeviceToHost, s->stream);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
-            if (e != cudaSuccess) { rc = cuda_status(e); break; }
-        } else {
-            if ((rc = enqueue_chunk(s, n))) break;
-            cudaError_t e = cudaMemcpyAsync(r, s->b.results, 4 * sizeof(double),
-                                            cudaMemcpyDeviceToHost, s->stream);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
-            if (e != cudaSuccess) { rc = cuda_status(e); break; }
-        }
+        if ((rc = graphs ? graph_chunk(s, n) : enqueue_chunk(s, n))) break;
+        rc = read_results(s, r);
+        if (rc && rc != LBM_ENONFINITE) break;
         du = r[1];
-        if ((rc = read_status(s))) break;
+        if (rc) break;
         if ((rc = refresh_scale(s))) break;
         rc = LBM_ENOTCONV;
         if (du < tol) { rc = LBM_OK; break; }
@@ -840,6 +836,27 @@ int lbm_moments(lbm_solver* s, double* rho, double* ux, double* uy) {
     if (!s) return LBM_EINVAL;
     const size_t n = size_t(s->Nx) * s->Ny * 8;
     cudaError_t e = cudaSuccess;
+    // a small channel's fields and its status lie within one short span of the
+    // workspace: one copy instead of four
+    char* const first = reinterpret_cast<char*>(s->b.rho);
+    const size_t span = size_t(reinterpret_cast<char*>(s->b.status) - first) + sizeof(unsigned);
+    if (rho && ux && uy && span <= kSmallRead) {
+        try {
+            s->readback.resize(span);
+        } catch (const std::bad_alloc&) {
+            return LBM_ENOMEM;
+        }
+        char* const h = s->readback.data();
+        e = cudaMemcpyAsync(h, first, span, cudaMemcpyDeviceToHost, s->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
+        if (e != cudaSuccess) return cuda_status(e);
+        std::memcpy(rho, h, n);
+        std::memcpy(ux, h + (reinterpret_cast<char*>(s->b.ux) - first), n);
+        std::memcpy(uy, h + (reinterpret_cast<char*>(s->b.uy) - first), n);
+        unsigned st = 0;
+        std::memcpy(&st, h + span - sizeof(st), sizeof(st));
+        return st ? LBM_ENONFINITE : LBM_OK;
+    }
     if (rho && e == cudaSuccess) e = cudaMemcpyAsync(rho, s->b.rho, n, cudaMemcpyDeviceToHost, s->stream);
     if (ux && e == cudaSuccess) e = cudaMemcpyAsync(ux, s->b.ux, n, cudaMemcpyDeviceToHost, s->stream);
     if (uy && e == cudaSuccess) e = cudaMemcpyAsync(uy, s->b.uy, n, cudaMemcpyDeviceToHost, s->stream);
@@ -851,21 +868,21 @@ int lbm_moments(lbm_solver* s, double* rho, double* ux, double* uy) {
 int lbm_mass_flow(lbm_solver* s, double* mdot, double* mean_ux) {
     if (!s) return LBM_EINVAL;
     double r[4];
-    int rc = reduce(s, false, r);
-    if (rc) return rc;
+    const int rc = reduce(s, false, r);
+    if (rc && rc != LBM_ENONFINITE) return rc;
     if (mdot) *mdot = r[3];
     if (mean_ux) *mean_ux = r[0];
-    return read_status(s);
+    return rc;
 }
 
 int lbm_slip_velocity(lbm_solver* s, double* us) {
     if (!s || !us) return LBM_EINVAL;
     if (s->Ny < 4) return LBM_EINVAL;
     double r[4];
-    int rc = reduce(s, false, r);
-    if (rc) return rc;
+    const int rc = reduce(s, false, r);
+    if (rc && rc != LBM_ENONFINITE) return rc;
     *us = r[2];
-    return read_status(s);
+    return rc;
 }
 
 int lbm_knudsen_layer(lbm_solver* s, double* uneq) {

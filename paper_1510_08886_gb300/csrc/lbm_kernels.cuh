@@ -1453,11 +1453,11 @@ cudaError_t launch_warp(const KParams<C>& k, int LP, const S* src, S* dst, const
 
 // Same step for any V <= LBM_MAX_V (R, P at run time).  The populations are
 // read twice (moment pass, relaxation pass); the second read hits L1/L2.
-// INIT = true builds the state from a density field instead of streaming:
-// fbar_a = rho0 w_a, then the same relaxation.
-template <int N, bool INIT, typename S, typename C>
+// INIT = true builds the state from a density field (rho0, or 1 everywhere)
+// instead of streaming: fbar_a = rho0 w_a, then the same relaxation.
+template <int N, bool INIT, typename S, typename C, int MV>
 __global__ void __launch_bounds__(kBlock)
-k_generic(const __grid_constant__ KParams<C> k, const S* src,
+k_generic(const __grid_constant__ KParams<C, MV> k, const S* src,
           const double* __restrict__ rho0, S* dst, const DevBufs b) {
     const int cell = blockIdx.x * kBlock + threadIdx.x;
     step_begin();
@@ -1468,7 +1468,7 @@ k_generic(const __grid_constant__ KParams<C> k, const S* src,
     C pb = C(0), pt = C(0);
     double r0 = 0.0;
     if (INIT) {
-        r0 = rho0[cell] - 1.0;
+        r0 = rho0 ? rho0[cell] - 1.0 : 0.0;
     } else {
         if (y < k.maxey) pb = C(wall_dpsi<S, C>(k, src, x, true));
         if (y >= k.Ny - k.maxey) pt = C(wall_dpsi<S, C>(k, src, x, false));
@@ -1540,7 +1540,7 @@ cudaError_t launch_step_n(const KParams<C>& k, const S* src, S* dst, const DevBu
         case 4: return LBM_STEP(SetD2V40);
         case 5: return LBM_STEP(SetD2V48);
         default:
-            return launch_chained(true, k_generic<N, false, S, C>, g, kBlock, 0, st, k, src,
+            return launch_chained(true, k_generic<N, false, S, C, LBM_MAX_V>, g, kBlock, 0, st, k, src,
                                   static_cast<const double*>(nullptr), dst, b);
     }
 #undef LBM_STEP
@@ -1578,13 +1578,24 @@ cudaError_t launch_init_t(const KParams<C>& k, int N, const double* rho0, void* 
                           const DevBufs& b, cudaStream_t st) {
     S* d = static_cast<S*>(dst);
     const dim3 g = grid_for(k);
+    // the smallest record that holds the set (see KParams)
+    auto go = [&](auto kernel, const auto& ks) {
+        kernel<<<g, kBlock, 0, st>>>(ks, nullptr, rho0, d, b);
+        return cudaGetLastError();
+    };
+#define LBM_INIT(NN)                                                                              \
+    case NN:                                                                                      \
+        return k.V <= 17   ? go(k_generic<NN, true, S, C, 17>, shrink_params<17>(k))              \
+               : k.V <= 33 ? go(k_generic<NN, true, S, C, 33>, shrink_params<33>(k))              \
+               : k.V <= 65 ? go(k_generic<NN, true, S, C, 65>, shrink_params<65>(k))              \
+                           : go(k_generic<NN, true, S, C, LBM_MAX_V>, k);
     switch (N) {
-        case 2: k_generic<2, true, S, C><<<g, kBlock, 0, st>>>(k, nullptr, rho0, d, b); break;
-        case 3: k_generic<3, true, S, C><<<g, kBlock, 0, st>>>(k, nullptr, rho0, d, b); break;
-        case 4: k_generic<4, true, S, C><<<g, kBlock, 0, st>>>(k, nullptr, rho0, d, b); break;
+        LBM_INIT(2)
+        LBM_INIT(3)
+        LBM_INIT(4)
         default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
+#undef LBM_INIT
 }
 
 }  // namespace lbm
