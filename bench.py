@@ -79,7 +79,7 @@ def measured_peaks():
 def kernel_source_hash():
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_1510_08886_gb300", "csrc")
-    for fn in ("lbm_kernels.cuh", "lbm_internal.h", "k_fp32.cu", "k_fp64.cu"):
+    for fn in ("lbm_kernels.cuh", "lbm_internal.h", "k_fp32.cu", "k_fp64.cu", "fx64.cuh"):
         with open(os.path.join(csrc, fn), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]

@@ -19,8 +19,14 @@
 //         with one fma: d* = (1 - omega) d + omega w G.
 //
 // Every rounding is to nearest or has zero mean: a bias of a fraction of a unit
-// per step would act on the flow like a body force.  Against a 113-bit
-// reference the result is closer than the FP64 evaluation's (fewer roundings).
+// per step would act on the flow like a body force.  Against a 113-bit reference
+// (random channel states, Kn 0.01 to 1, u 1e-3 to 3e-2) the rms error of a node's
+// post-collision moments relative to the FP64 evaluation's is 0.8 to 1.1 in the
+// density, 0.25 to 1.0 in x and 0.5 to 1.1 in y momentum.
+//
+// Per 32 nodes and step (D2V33, N = 4) this issues 3670 instructions, 33 of them
+// FP64, against ~475 FP64 ones of 64 cycles: 334 us per step on 4096 x 512 (1586),
+// D2V16 163 us (12.8 GLUPS), D2V53 2048 x 512 303 us.
 //
 // Nodes outside the range of the fixed-point form (a density far from 1, a flow
 // speed near the lattice's limit, non-finite values) and solves whose force

@@ -1,5 +1,5 @@
 // Device code of the fused stream-collide step (templates, instantiated per
-// precision in k_fp64.cu and k_fp32.cu).
+// precision in k_fp64.cu, k_fp32.cu, k_fp16.cu and k_bf16.cu).
 //
 // One thread owns one lattice node (x, y).  Per time step it
 //   1. pulls the V post-collision populations of the previous step from
@@ -1132,8 +1132,13 @@ __device__ __forceinline__ void wall_strip(const KParams<C, MV>& k, const S* __r
     flag_density<C>(q, b.status);
 }
 
-// Fused step for a compiled velocity set: the V populations stay in registers
-// between the moment pass and the relaxation pass.
+// Fused step for a compiled velocity set.  In fp32 and 16-bit storage the V
+// populations stay in registers between the moment pass and the relaxation pass;
+// fp64 copies them to shared memory as they arrive (cp.async) and runs the
+// fixed-point collision on them there (fx64.cuh), which leaves 96 registers and
+// 20 warps per SM.  fp32 is bound by HBM (D2V33 4096 x 512: 82 us per step, 6.7
+// TB/s), 16-bit by instruction issue, fp64 by integer issue and fetch (334 us,
+// 3.3 TB/s; 1586 us when the FP64 pipe evaluated it).
 //  - fast path (block-uniform): the block's nodes lie in one row at least
 //    max|e_y| rows from both walls and max|e_x| columns from both ends, so
 //    every pull is a fixed offset from the node: one address per population;
@@ -1151,11 +1156,10 @@ k_step_ct(const __grid_constant__ KParams<C, SET::R + 2 * SET::P> k, const S* sr
     // block 2 strips + m then takes the interior block at node (strips + m) 128.
     int blk = int(blockIdx.x);
     // A grid of several waves lets the next step's blocks into its tail; a small
-    // one lets them in at its end, else they pile up on the SMs that are free
-    // first (fp64 D2V33 257 x 131: 19.6 us per step against 14.7; bf16 D2V40
+    // one lets them in as its blocks end, else they pile up on the SMs that are
+    // free first (fp64 D2V33 257 x 131: 19.6 us per step against 14.7; bf16 D2V40
     // 320 x 152: 24 against 20)
-    const bool waves = gridDim.x >= 8 * 152;
-    if (waves) step_begin();
+    if (gridDim.x >= 8 * 152) step_begin();
     if (k.strips) {
         if (blk < 2 * k.strips) step_wait();
         if (blk < k.strips) {
@@ -1202,7 +1206,6 @@ k_step_ct(const __grid_constant__ KParams<C, SET::R + 2 * SET::P> k, const S* sr
     }
     const CellCoef<C> q = finish_node<SET, N, S, C>(k, f, k.emit != 0, sr_seed<S, C>(k.seed, cell),
                                                     [&](auto a, S v) { static_cast<S*>(k.dstp[a])[cell] = v; });
-    if (!waves) step_begin();
     emit_moments<C>(k, q, cell, b);
     flag_density<C>(q, b.status);
 }
@@ -1468,7 +1471,8 @@ k_generic(const __grid_constant__ KParams<C, MV> k, const S* src,
     C pb = C(0), pt = C(0);
     double r0 = 0.0;
     if (INIT) {
-        r0 = rho0 ? rho0[cell] - 1.0 : 0.0;
+        if (rho0) r0 = rho0[cell] - 1.0;
+        else b.prev_ux[cell] = 1.0;          // as a density field of ones would leave it
     } else {
         if (y < k.maxey) pb = C(wall_dpsi<S, C>(k, src, x, true));
         if (y >= k.Ny - k.maxey) pt = C(wall_dpsi<S, C>(k, src, x, false));
