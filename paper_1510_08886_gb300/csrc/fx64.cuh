@@ -84,6 +84,7 @@ constexpr int kMaxRows = 32;
 //   theta A_xx / 2 = k1 K_xx - k0 drho + k2 rho X^2 / 2 + k3 M_x, ...
 struct Consts {
     int ok;                  // 1: the fixed-point form may be used
+    int mirror;              // 1: g < 0, the constants are those of |g|
     int emin;                // least E: keeps h and theta in range
     int h_exp, th_exp;       // h = h_m 2^-h_exp, theta = th_m 2^-th_exp
     i64 h_m, th_m;           // 62-bit mantissas; h = c (dt/2) g
@@ -101,6 +102,7 @@ struct Consts {
     int nx, ny, nd, rest;    // rest: 1 if plane 0 is the rest population
     Mul om0;                 // omega w of the rest population = om0 2^-oe0
     int oe0, fam;            // fam: see FamilyFormat, -1: none fits
+    int pad;
     Row row[kMaxRows];
     // per pair (plane order): omega w = pom 2^-poe
     Mul pom[kMaxRows];
@@ -331,7 +333,12 @@ LBM_HD i64 const_q(i64 mant, int exp, int q, unsigned& frac) {
 // a = rho X^4 / 4 (and the mixed products).  Shifts left before a product use
 // the room the bounds leave, so that a product loses less than a unit.
 template <class FMT, int N, bool FORCE>
-LBM_HD bool coefs(const Consts& k, const Sums& m, int E, Poly& p) {
+LBM_HD bool coefs(const Consts& k, Sums m, int E, Poly& p) {
+    // g < 0 is the mirror image in x of |g|: e_x -> -e_x before and after
+    if (FORCE && k.mirror) {
+        m.jx = -m.jx;
+        m.kxy = -m.kxy;
+    }
     constexpr int S2 = FMT::S2, S3 = FMT::S3, C2 = FMT::C2;
     const int q = 1074 + FMT::S0 - E;
     const float fd = hif(m.d), fj = fabsf_(hif(m.jx)) + fabsf_(hif(m.jy));
@@ -426,6 +433,18 @@ LBM_HD bool coefs(const Consts& k, const Sums& m, int E, Poly& p) {
             p.d30 += mulc(shl(axx, 64 - C2 + S3), k.c2);
             p.d21 += mulc(shl(axy, 65 - C2 + S3), k.c2);
             p.d12 += mulc(shl(ayy, 64 - C2 + S3), k.c2);
+        }
+    }
+    if (FORCE && k.mirror) {
+        p.c11 = -p.c11;
+        p.d10 = -p.d10;
+        if (N >= 3) {
+            p.d30 = -p.d30;
+            p.d12 = -p.d12;
+        }
+        if (N >= 4) {
+            p.c31 = -p.c31;
+            p.c13 = -p.c13;
         }
     }
     return ok && bound < 1.9e9f;
@@ -642,7 +661,7 @@ LBM_CX SetInfo set_info() {
 // Host: the constants of a solve (lattice speed c, relaxation time tau, time
 // step dt, force g along x) of a set with planes e = (ex, ey), weights w, the
 // rest plane first if R = 1, then P pair members and their negatives.  ok = 0 if
-// a constant leaves its range (very large forces or Knudsen numbers, g < 0).
+// a constant leaves its range (very large forces or Knudsen numbers).
 inline Mul to_mul(long double v, int point, int& ok) {
     const long double x = ldexpl(v, point);
     if (!(x >= 0.0L && x < 4611686018427387904.0L)) { ok = 0; return Mul{0, 0, 0}; }
@@ -662,9 +681,9 @@ inline Consts make_consts(double c_, double tau_, double dt_, double g_, int R, 
     const int emax = si.emax, ks = si.ks;
     Consts k;
     memset(&k, 0, sizeof(k));
-    // the theta terms carry the sign of g; only g >= 0 has the fixed-point form
-    if (!(g_ >= 0.0) || emax < 1) return k;
-    const long double c = c_, tau = tau_, dt = dt_, g = g_;
+    if (emax < 1) return k;
+    const long double c = c_, tau = tau_, dt = dt_, g = fabs(g_);
+    k.mirror = g_ < 0.0;
     const long double h = 0.5L * dt * g * c, th = tau * c * g, k2t = 1.0L / (2 * tau + dt);
     k.ok = 1;
     k.emin = 128;

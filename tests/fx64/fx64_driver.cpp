@@ -61,7 +61,7 @@ static int run(const char* name, double c, int tries) {
         for (int t = 0; t < tries; ++t) {
             const double Kn = std::pow(10.0, unif(-2, regime ? 1 : 0)), Ny = std::floor(unif(16, 2048));
             const double tau = std::sqrt(2 / M_PI) * Kn, dt = 1 / (Ny * c);
-            const double g = FORCE ? 8 * tau * std::pow(10.0, unif(-4, regime ? -1 : -2)) : 0.0;
+            const double g = FORCE ? (t % 2 ? -8 : 8) * tau * std::pow(10.0, unif(-4, regime ? -1 : -2)) : 0.0;
             const double omega = dt / (tau + 0.5 * dt), omo = 1 - omega;
             const fx::Consts k = fx::make_consts(c, tau, dt, g, SET::R, SET::P, ex.data(), ey.data(), w.data(),
                                                  fx::set_info<SET>());

@@ -77,3 +77,10 @@ def test_small_channels_on_lanes(name, N, Nx, Ny, amplitude, mach):
     """Several lanes per node, resident on a cluster of small or large blocks;
     the second flow takes the general form on some nodes of a warp."""
     _compare(name, N, Nx, Ny, 7, amplitude=amplitude, mach=mach)
+
+
+@pytest.mark.parametrize("name,N", [("D2V33", 4), ("D3V107xz", 3)])
+@pytest.mark.parametrize("Nx,Ny", [(129, 60), (4, 40)])
+def test_force_against_x(name, N, Nx, Ny):
+    """g < 0 runs as the mirror image of g > 0."""
+    _compare(name, N, Nx, Ny, 7, mach=-1e-2)
