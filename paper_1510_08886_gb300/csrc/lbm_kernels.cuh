@@ -35,7 +35,10 @@ namespace lbm {
 // next step's blocks take the slots this step leaves free and compute their
 // indices there; step_wait, before the first access to a lattice or a moment
 // field, returns when every earlier step has completed and its stores are
-// visible.  (Without the launch attribute both do nothing.)
+// visible.  (Without the launch attribute both do nothing.)  Pointers to a lattice
+// carry no __restrict__, in the kernels and in their helpers: const __restrict__
+// would allow the read-only load path, whose data are taken to be constant for
+// the whole life of the kernel, and here the last step may still write them.
 __device__ __forceinline__ void step_begin() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void step_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -240,7 +243,7 @@ __device__ __forceinline__ double wall_dpsi_by(const KParams<C, MV>& k, int x, b
 
 // The same sum read from a lattice in global memory ([V][Ny][Nx] planes).
 template <typename S, typename C, int MV>
-__device__ __noinline__ double wall_dpsi(const KParams<C, MV>& k, const S* __restrict__ src, int x,
+__device__ __noinline__ double wall_dpsi(const KParams<C, MV>& k, const S* src, int x,
                                          bool bottom) {
     return wall_dpsi_by<S, C>(k, x, bottom, [&](int b, int row, int xs) {
         return src[(long long)b * k.plane + (long long)row * k.Nx + xs];
@@ -312,7 +315,7 @@ __device__ __forceinline__ double wall_sum_ct(const TERM& term, std::integer_seq
 
 // Wall balance of a compiled set on a lattice in device memory.
 template <class SET, typename S, typename C, bool BOTTOM, int MV>
-__device__ __forceinline__ double wall_dpsi_ct(const KParams<C, MV>& k, const S* __restrict__ src, int x) {
+__device__ __forceinline__ double wall_dpsi_ct(const KParams<C, MV>& k, const S* src, int x) {
     constexpr int V = SET::R + 2 * SET::P;
     auto term = [&](auto bc, int j) {
         constexpr int b = decltype(bc)::value;
@@ -483,7 +486,7 @@ __device__ __forceinline__ void emit_moments(const KParams<C, MV>& k, const Cell
 
 // Pull one population of plane a into node (x, y) of an interior row.
 template <typename S, typename C, int MV>
-__device__ __forceinline__ C pull(const KParams<C, MV>& k, const S* __restrict__ src, int a, int x, int y) {
+__device__ __forceinline__ C pull(const KParams<C, MV>& k, const S* src, int a, int x, int y) {
     int xs = x - k.sx[a];
     xs += (xs < 0) ? k.Nx : 0;
     return ld_pop<S, C>(k, src[(long long)a * k.plane + (long long)(y - k.ey[a]) * k.Nx + xs], a);
@@ -492,7 +495,7 @@ __device__ __forceinline__ C pull(const KParams<C, MV>& k, const S* __restrict__
 // Populations of a wall node of a compiled set: the fill for those whose
 // source lies beyond a wall, the pull for the others.
 template <class SET, typename S, typename C, int A, int MV>
-__device__ __forceinline__ C wall_value(const KParams<C, MV>& k, const S* __restrict__ src, int x, int y,
+__device__ __forceinline__ C wall_value(const KParams<C, MV>& k, const S* src, int x, int y,
                                         C pb, C pt) {
     constexpr int EY = A < SET::R ? 0 : (A < SET::R + SET::P ? SET::ey[A - SET::R] : -SET::ey[A - SET::R - SET::P]);
     const int ys = y - EY;
@@ -513,7 +516,7 @@ __host__ __device__ constexpr int plane_ey_ct(int a) {
 // given: the fill where the source lies beyond that wall, the pull otherwise
 // (the other wall is out of reach, Ny >= 8).
 template <class SET, typename S, typename C, bool BOTTOM, int A, int MV>
-__device__ __forceinline__ C strip_value(const KParams<C, MV>& k, const S* __restrict__ src, int x, int y,
+__device__ __forceinline__ C strip_value(const KParams<C, MV>& k, const S* src, int x, int y,
                                          C dpsi) {
     constexpr int EY = plane_ey_ct<SET>(A);
     const int ys = y - EY;
@@ -524,7 +527,7 @@ __device__ __forceinline__ C strip_value(const KParams<C, MV>& k, const S* __res
 }
 
 template <class SET, typename S, typename C, bool BOTTOM, int MV, int... I>
-__device__ __forceinline__ void strip_values(const KParams<C, MV>& k, const S* __restrict__ src, int x, int y,
+__device__ __forceinline__ void strip_values(const KParams<C, MV>& k, const S* src, int x, int y,
                                              C dpsi, C* f, std::integer_sequence<int, I...>) {
     ((f[I] = strip_value<SET, S, C, BOTTOM, I>(k, src, x, y, dpsi)), ...);
 }
@@ -937,7 +940,7 @@ __device__ __forceinline__ double* step_scratch() {
 }
 
 // Copy one population to the scratch without passing a register.
-__device__ __forceinline__ void copy_async(double* dst, const double* __restrict__ src) {
+__device__ __forceinline__ void copy_async(double* dst, const double* src) {
     const unsigned d = unsigned(__cvta_generic_to_shared(dst));
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
 }
@@ -994,7 +997,7 @@ __device__ __forceinline__ CellCoef<C> finish_node(const KParams<C, MV>& k, C* f
 // dPsi given (pb bottom, pt top; 0 where out of reach): the fill where the
 // source lies beyond a wall, the pull otherwise.
 template <int MV>
-__device__ __forceinline__ void take_wall64(const KParams<double, MV>& k, const double* __restrict__ src, int x,
+__device__ __forceinline__ void take_wall64(const KParams<double, MV>& k, const double* src, int x,
                                             int y, double pb, double pt) {
     double* sf = step_scratch();
 #pragma unroll 4
@@ -1012,7 +1015,7 @@ __device__ __forceinline__ void take_wall64(const KParams<double, MV>& k, const 
 
 // Populations of a wall node of a compiled set (registers f; fp64: the scratch).
 template <class SET, typename S, typename C, int MV, int... I>
-__device__ __forceinline__ void pull_wall_ct(const KParams<C, MV>& k, const S* __restrict__ src, int x,
+__device__ __forceinline__ void pull_wall_ct(const KParams<C, MV>& k, const S* src, int x,
                                              int y, C* f, std::integer_sequence<int, I...>) {
     const C pb = y < k.maxey ? C(wall_dpsi_ct<SET, S, C, true>(k, src, x)) : C(0);
     const C pt = y >= k.Ny - k.maxey ? C(wall_dpsi_ct<SET, S, C, false>(k, src, x)) : C(0);
@@ -1096,7 +1099,7 @@ __device__ __forceinline__ double strip_partial(const TERM& term, std::integer_s
 }
 
 template <class SET, int N, typename S, typename C, bool BOTTOM, int MV>
-__device__ __forceinline__ void wall_strip(const KParams<C, MV>& k, const S* __restrict__ src, int strip,
+__device__ __forceinline__ void wall_strip(const KParams<C, MV>& k, const S* src, int strip,
                                            const DevBufs& b) {
     constexpr int R = SET::R, P = SET::P, V = R + 2 * P;
     __shared__ double part[4][32];
