@@ -319,12 +319,13 @@ LBM_HD int f2i(float x) {
 }
 
 // The per-solve constant mant 2^-exp in the unit 2^-q: integer part and the
-// 32 bits below it.
+// 32 bits below it, whatever lies below those cut (a force of 2^-33 units of one
+// node's sums is none).
 LBM_HD i64 const_q(i64 mant, int exp, int q, unsigned& frac) {
-    int sh = exp - q;
-    sh = sh < 63 ? sh : 63;                                // >= 2 (emin)
-    frac = unsigned(u64(mant << (64 - sh)) >> 32);
-    return mant >> sh;
+    int sh = exp - q;                                      // >= 2 (emin)
+    sh = sh < 95 ? sh : 95;
+    frac = unsigned(sh < 32 ? u64(mant) << (32 - sh) : u64(mant) >> (sh - 32));
+    return mant >> (sh < 63 ? sh : 63);
 }
 
 // Target coefficients from the sums; false outside the fixed-point range.
