@@ -193,7 +193,7 @@ template <int S0>
 LBM_HD i64 to_fixed(double d, int E) {
     const int hi = dhi(d);
     const unsigned lo = dlo(d);
-    const int sh = E - ((hi >> 20) & 0x7ff);           // 0 .. 1021
+    const int sh = E - ((hi >> 20) & 0x7ff);           // 0 .. kLargestE
     const int s = hi >> 31;
     int xh = int((unsigned(hi) << S0) | (lo >> (32 - S0)));
     xh = ((xh & ((1 << (20 + S0)) - 1)) | (1 << (20 + S0))) ^ s;
@@ -203,7 +203,8 @@ LBM_HD i64 to_fixed(double d, int E) {
     return i64(u64(y + 1) & ~u64(1));
 }
 
-// T 2^(eb - 1084) as a double, rounded to nearest; |T| < 2^62.
+// T 2^(eb - 1084) as a double, rounded to nearest; |T| < 2^62 (T = 0: a quarter of
+// the unit).
 LBM_HD double to_double(i64 T, int eb) {
     const int s = int(T >> 63);
     const u64 a = u64((T ^ i64(s)) - i64(s));
@@ -271,6 +272,11 @@ struct FamilyFormat {
 struct Sums {
     i64 d, jx, jy, kxx, kxy, kyy;
 };
+
+// Range of E.  Below: populations this small (2^-895) are those of a fluid at rest
+// without a force, whose zeros the FP64 form keeps; to_double has none.
+constexpr int kLeastE = 128, kLargestE = 1021;
+LBM_HD bool exponent_fits(int E) { return E > kLeastE && E <= kLargestE; }
 
 // exponent key of |e| d, lg = log2 of |e|
 LBM_HD unsigned key(double d, int lg) { return (unsigned(dhi(d)) & 0x7fffffffu) + (unsigned(lg) << 20); }
@@ -544,7 +550,7 @@ LBM_HD bool collide(const Consts& k, double omo, Sums& m, int& E, const GET& get
         t = umax_(t, umax_(key(get(w.b, w.bm, -w.ax, w.ay), w.lg), key(get(w.bm, w.b, w.ax, -w.ay), w.lg)));
     });
     E = int(t >> 20);
-    if (E > 1021) return false;
+    if (!exponent_fits(E)) return false;
     phase();
     m = Sums{0, 0, 0, 0, 0, 0};
     if constexpr (SET::R != 0) m.d = to_fixed<S0>(get(0, 0, 0, 0), E);
@@ -687,7 +693,7 @@ inline Consts make_consts(double c_, double tau_, double dt_, double g_, int R, 
     k.mirror = g_ < 0.0;
     const long double h = 0.5L * dt * g * c, th = tau * c * g, k2t = 1.0L / (2 * tau + dt);
     k.ok = 1;
-    k.emin = 128;
+    k.emin = kLeastE;
     for (int i = 0; i < 2; ++i) {
         const long double v = i ? th : h;
         int e = 0;
@@ -703,7 +709,7 @@ inline Consts make_consts(double c_, double tau_, double dt_, double g_, int R, 
     }
     // the rounding of the sums K enters the odd coefficients times theta c^4 e^3:
     // harmless for theta < 1/8 (8 tau^2 c Ma: Kn up to 4 at Ma = 1e-3)
-    if (k.emin > 1021 || th >= 0.125L) k.ok = 0;
+    if (k.emin > kLargestE || th >= 0.125L) k.ok = 0;
     k.c2 = to_mul(c * c, c2_point(emax), k.ok);
     k.h_63 = to_mul(h, 63, k.ok);
     k.th_63 = to_mul(th, 63, k.ok);

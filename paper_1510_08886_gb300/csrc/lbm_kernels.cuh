@@ -1332,7 +1332,7 @@ __device__ __forceinline__ CellCoef<double> warp_node_fx(const KParams<double, M
     const int E = int(t >> 20);
     CellCoef<double> q{};
     // (out of range: any E will do, the result is not used)
-    const int Es = min(E, 1021);
+    const int Es = min(E, fx::kLargestE);
     const long long vp = fx::to_fixed<S0>(fp, Es), vm = fx::to_fixed<S0>(fm, Es);
     const long long sum = vp + vm, dif = vp - vm;
     const long long ks = (sum + (1ll << FMT::KS >> 1)) >> FMT::KS;
@@ -1342,7 +1342,7 @@ __device__ __forceinline__ CellCoef<double> warp_node_fx(const KParams<double, M
     node_sum6<LP, long long>(m, p);
     const fx::Sums s{m[0], m[1], m[2], m[3], m[4], m[5]};
     fx::Poly c;
-    ok = E <= 1021 && fx::coefs<FMT, N, FORCE>(k.fx, s, Es, c);
+    ok = fx::exponent_fits(E) && fx::coefs<FMT, N, FORCE>(k.fx, s, Es, c);
     if (!ok || !node) return q;
     const int eb = Es + 10 + 64 - S0;
     if (act) {
