@@ -675,11 +675,13 @@ inline Mul to_mul(long double v, int point, int& ok) {
     return make_mul(i64(rintl(x)));
 }
 
-// omega w = m 2^-oe with m in [2^61, 2^62)
+// omega w = m 2^-oe with m in [2^61, 2^62).  A target's biased exponent is at least
+// E + 69 - oe - 62 (relax): oe may not exceed the least E by more than 6.
 inline Mul to_weight(double ow, int& oe, int& ok) {
     int e = 0;
     frexp(ow, &e);
     oe = 62 - e;
+    if (oe > kLeastE + 7) ok = 0;
     return to_mul(ow, oe, ok);
 }
 
