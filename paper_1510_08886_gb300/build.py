@@ -21,6 +21,9 @@ SOURCES = ["k_fp64.cu", "k_cluster.cu", "k_fp32.cu", "k_fp16.cu", "k_bf16.cu", "
            "engine_fp64.cu", "engine_res_fp64.cu",
            "engine_bf16.cu", "engine_res_fp32.cu", "engine_res_half.cu", "engine_res_bf16.cu",
            "lbm_engine.cu", "lbm_api.cu", "lbm_noalloc.cu", "peak_probe.cu", "dvm.cpp", "dvm_gen.cpp"]
+# sources compiled once more per velocity set, with this macro naming the set
+PER_SET = {"engine_res_fp64.cu": "LBM_RES_SET"}
+SETS = ["SetD2V53", "SetD2V48", "SetD2V40", "SetD2V33", "SetD2V32", "SetD2V16"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -47,9 +50,14 @@ def build(force=False, verbose=False):
     if verbose:
         common += ["-Xptxas", "-v"]
 
-    def compile_one(src):
-        obj = os.path.join(OUT, os.path.splitext(src)[0] + ".o")
-        cmd = [nvcc] + common + ["-c", os.path.join(CSRC, src), "-o", obj]
+    # the longest first
+    units = [(src, f"-D{macro}={s}", "_" + s) for src, macro in PER_SET.items() for s in SETS]
+    units += [(src, None, "") for src in SOURCES]
+
+    def compile_one(unit):
+        src, define, suffix = unit
+        obj = os.path.join(OUT, os.path.splitext(src)[0] + suffix + ".o")
+        cmd = [nvcc] + common + ([define] if define else []) + ["-c", os.path.join(CSRC, src), "-o", obj]
         if src.endswith(".cpp"):
             cmd = [nvcc, "-O2", "-std=c++17", "-Xcompiler", "-fPIC", "-I", INCLUDE, "-c",
                    os.path.join(CSRC, src), "-o", obj]
@@ -58,8 +66,8 @@ def build(force=False, verbose=False):
             raise RuntimeError(f"nvcc failed for {src}:\n{r.stdout}\n{r.stderr}")
         return obj, r.stderr
 
-    with cf.ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:
-        results = list(ex.map(compile_one, SOURCES))
+    with cf.ThreadPoolExecutor(max_workers=len(units)) as ex:
+        results = list(ex.map(compile_one, units))
     if verbose:
         for _, log in results:
             sys.stderr.write(log)
