@@ -96,13 +96,13 @@ struct Consts {
     Mul k0_63;               // theta k / 2                   (times drho)
     Mul k2_60;               // theta dt / ((2 tau + dt) c^2) (times S / 2)
     Mul k3_62, k3h_62;       // theta tau g dt / ((2 tau + dt) c) and its half (times M)
-    float gj, ga;            // bound on |G| and its partial sums from the high words of J and theta A
+    float gm, ga;            // bound on |G| and its partial sums from the high words of M and theta A
+    float em;                // max |e|: the same from theta
     float xlim, c2f;         // bound on |X| + |Y|; c^2
     // rows [0, nx): e = (ax, 0); [nx, ny): (0, ay); [ny, nd): four velocities
     int nx, ny, nd, rest;    // rest: 1 if plane 0 is the rest population
     Mul om0;                 // omega w of the rest population = om0 2^-oe0
     int oe0, fam;            // fam: see FamilyFormat, -1: none fits
-    int pad;
     Row row[kMaxRows];
     // per pair (plane order): omega w = pom 2^-poe
     Mul pom[kMaxRows];
@@ -334,6 +334,8 @@ LBM_HD i64 const_q(i64 mant, int exp, int q, unsigned& frac) {
     return mant >> (sh < 63 ? sh : 63);
 }
 
+constexpr float kGMax = 1.9e9f;      // of the high word of G: |G| < 2^62.9
+
 // Target coefficients from the sums; false outside the fixed-point range.
 // Binary points: U_G = 2^-q with q = 1074 + S0 - E; X, Y = c u and eps = drho / rho
 // are multiples of 2^-62.  M = rho X, H = rho X X / 2, t = rho X X X / 2,
@@ -353,16 +355,21 @@ LBM_HD bool coefs(const Consts& k, Sums m, int E, Poly& p) {
     if (FORCE && N >= 3) fk = fabsf_(hif(m.kxx)) + fabsf_(hif(m.kxy)) + fabsf_(hif(m.kyy));
     const float un = exp2i(q < 150 ? 31 - q : -119);       // high word of a sum -> its value
     const float delta = fd * un;
-    const float bound = k.gj * fj + fabsf_(fd);
-    bool ok = fj < (C2 == 61 ? 5.0e8f : 1.9e9f) && fk < 5.0e8f && k.c2f * fj * un < k.xlim &&
-              delta > -0.4f && delta < 1.9f;
-
     unsigned hfrac = 0u, tfrac = 0u;
     i64 hq = 0, tq = 0;
+    // bounds on |M| (high word, and as a value: |X| + |Y|) and |G|
+    float fm = 0.5f * k.c2f * fj, bound = fabsf_(fd);
     if (FORCE) {
         hq = const_q(k.h_m, k.h_exp, q, hfrac);
         tq = const_q(k.th_m, k.th_exp, q, tfrac);
+        const float rho = 1.0f + delta;
+        fm += rho * hif(hq);
+        bound += rho * k.em * hif(tq);
     }
+    bound += k.gm * fm;
+    bool ok = fj < (C2 == 61 ? 5.0e8f : 1.9e9f) && fk < 5.0e8f && 2.0f * fm * un < k.xlim &&
+              delta > -0.4f && delta < 1.9f;
+
     i64 Mx = mulc(shl(m.jx, 63 - C2), k.c2, hfrac);
     const i64 My = mulc(shl(m.jy, 63 - C2), k.c2);
     if (FORCE) Mx += hq + mulc(m.d, k.h_63);
@@ -434,7 +441,7 @@ LBM_HD bool coefs(const Consts& k, Sums m, int E, Poly& p) {
             const i64 axx = mulc(shl(m.kxx, 2), k.k1) - kd + mulc(shl(Hxx, 4 - S2), k.k2_60) + mulc(Mx2, k.k3_62);
             const i64 axy = mulc(shl(m.kxy, 2), k.k1) + mulc(sh_(Sxy, 3 - S2), k.k2_60) + mulc(My2, k.k3h_62);
             const i64 ayy = mulc(shl(m.kyy, 2), k.k1) - kd + mulc(shl(Hyy, 4 - S2), k.k2_60);
-            ok = ok && k.ga * (fabsf_(hif(axx)) + fabsf_(hif(axy)) + fabsf_(hif(ayy))) + bound < 1.9e9f;
+            ok = ok && k.ga * (fabsf_(hif(axx)) + fabsf_(hif(axy)) + fabsf_(hif(ayy))) + bound < kGMax;
             p.d10 -= 3 * axx + ayy;
             p.d01 -= 2 * axy;
             p.d30 += mulc(shl(axx, 64 - C2 + S3), k.c2);
@@ -454,7 +461,7 @@ LBM_HD bool coefs(const Consts& k, Sums m, int E, Poly& p) {
             p.c13 = -p.c13;
         }
     }
-    return ok && bound < 1.9e9f;
+    return ok && bound < kGMax;
 }
 
 // d* = (1 - omega) d + T, T = G omega w already scaled (units 2^(eb - 1084))
@@ -723,9 +730,10 @@ inline Consts make_consts(double c_, double tau_, double dt_, double g_, int R, 
     k.k2_60 = to_mul(th * dt * k2t / (c * c), 60, k.ok);
     k.k3_62 = to_mul(th * tau * g * dt * k2t / c, 62, k.ok);
     k.k3h_62 = to_mul(0.5L * th * tau * g * dt * k2t / c, 62, k.ok);
-    // s = c u.e stays below 0.4, so |G| < |drho| + 1.3 s + ..., the sums of
-    // second order stay below 0.25 s and those of third order below 0.04 s (in
-    // units with extra bits), besides the theta M e^2 and theta A e^3 terms
+    // M.e stays below 0.4 (xlim; the force's part h rho counts), so |G| < |drho| +
+    // 1.3 M.e + theta rho e_x + ..., the sums of second order stay below 0.25 M.e and
+    // those of third order below 0.04 M.e (in units with extra bits), besides the
+    // theta M e^2 and theta A e^3 terms
     const float em = float(emax), f2 = float(1 << extra2(emax)), f3 = float(1 << extra3(emax));
     const float te = 2.0f * float(th) * em;
     float gj = 1.35f + te;
@@ -733,7 +741,12 @@ inline Consts make_consts(double c_, double tau_, double dt_, double g_, int R, 
     if (f3 * 0.05f > gj) gj = f3 * 0.05f;
     k.xlim = 0.4f / em;
     k.c2f = float(c * c);
-    k.gj = 0.5f * k.c2f * em * gj;
+    // M is shifted left by 2 + s2 bits before a product: |M| < 2^59 with the extra
+    // bits, 2^61 without (a uniform flow's is at most 2^57.6 and 2^58.8 U_G in the
+    // paper's sets)
+    const float room = extra2(emax) ? 1.3e8f : 5.2e8f;
+    k.gm = em * gj > kGMax / room ? em * gj : kGMax / room;
+    k.em = em;
     k.ga = f3 * (4.0f + 4.0f * k.c2f * em * em) * em;
     const double omega = dt_ / (tau_ + 0.5 * dt_);
     k.rest = R;
