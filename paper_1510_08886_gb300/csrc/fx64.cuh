@@ -397,7 +397,9 @@ LBM_HD bool coefs(const Consts& k, Sums m, int E, Poly& p) {
     }
     const MulV xm = mulv(X), ym = mulv(Y);
     // H, S and a in units 2^-S2 U_G, t in units 2^-S3 U_G
-    const i64 Hxx = mulx(shl(Mx, 1 + S2), xm), Sxy = mulx(shl(Mx, 2 + S2), ym), Hyy = mulx(shl(My, 1 + S2), ym);
+    // (Sxy with the extra bits: 2 Y instead of a shift that M has no room for)
+    const i64 Hxx = mulx(shl(Mx, 1 + S2), xm), Hyy = mulx(shl(My, 1 + S2), ym);
+    const i64 Sxy = S2 ? mulx(shl(Mx, 1 + S2), mulv(shl(Y, 1))) : mulx(shl(Mx, 2), ym);
     p.c00 = dG - shl(mulc(shl(Hxx + Hyy, 5 - S2), k.ic4_60), 1);
     p.c20 = Hxx;
     p.c11 = Sxy;
@@ -741,10 +743,9 @@ inline Consts make_consts(double c_, double tau_, double dt_, double g_, int R, 
     if (f3 * 0.05f > gj) gj = f3 * 0.05f;
     k.xlim = 0.4f / em;
     k.c2f = float(c * c);
-    // M is shifted left by 2 + s2 bits before a product: |M| < 2^59 with the extra
-    // bits, 2^61 without (a uniform flow's is at most 2^57.6 and 2^58.8 U_G in the
-    // paper's sets)
-    const float room = extra2(emax) ? 1.3e8f : 5.2e8f;
+    // M is shifted left by 3 bits with the extra bits, by 2 without, before a product:
+    // |M| < 2^60 or 2^61 (a uniform flow's is at most 2^58.8 U_G in the paper's sets)
+    const float room = extra2(emax) ? 2.6e8f : 5.2e8f;
     k.gm = em * gj > kGMax / room ? em * gj : kGMax / room;
     k.em = em;
     k.ga = f3 * (4.0f + 4.0f * k.c2f * em * em) * em;
