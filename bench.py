@@ -32,9 +32,6 @@ sys.path.insert(0, ROOT)
 import numpy as np  # noqa: E402
 
 METRIC = "GLUPS & %HBM roofline"
-# algorithmic fp64 operations of one node update: ~20 V after pairing the +-e
-# populations (moments, equilibrium and force of each pair evaluated once)
-FP64_FLOPS_PER_NODE_PER_V = 20
 UNIT = "GLUPS"
 DVM, ORDER, NX, NY, SEED = "D2V33", 4, 4096, 512, 20151029
 WORKLOAD = ("channel D2V33 (S^{D2V33}_{Q9E132}), Hermite order 4, Nx=4096 periodic x "
@@ -97,6 +94,14 @@ def ncu_traffic(precision):
     if not m or not hsh or hsh.group(1) != kernel_source_hash():
         return None
     return float(m.group(1))
+
+
+def step_roofline(achieved, peak, peak_kind, traffic):
+    """Bytes that a step cannot do without per second against the HBM rate, in
+    every precision: no arithmetic pipe bounds the step (the fp64 collision runs
+    on the integer pipes)."""
+    return {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
+            "traffic": traffic, "peak_kind": peak_kind}
 
 
 class ClockSampler:
@@ -640,19 +645,7 @@ def main():
     peak, peak_kind = measured_peaks()
     achieved = bytes_per_launch / avg_launch_s / 1e9
     traffic = ncu_traffic(args.precision)
-    if args.precision != "fp64":
-        roofline = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                    "frac": achieved / peak, "traffic": traffic, "peak_kind": peak_kind}
-    else:
-        # fp64: bound by GB300's fp64 pipe; the peak is measured live (FMA chains
-        # on every SM, lbm_fma_rate), the flops are the algorithmic 20 V per node
-        flops = FP64_FLOPS_PER_NODE_PER_V * V * ncell / avg_launch_s / 1e12
-        alu_peak = lbm.fma_rate("fp64", stream) / 1e12
-        roofline = {"bound": "alu", "achieved": flops, "peak": alu_peak, "unit": "TFLOP/s",
-                    "frac": flops / alu_peak, "traffic": traffic,
-                    "peak_kind": "measured: independent DFMA chains on every SM (lbm_fma_rate)",
-                    "flops_per_node": FP64_FLOPS_PER_NODE_PER_V * V,
-                    "hbm_achieved_GBs": achieved, "hbm_frac": achieved / peak}
+    roofline = step_roofline(achieved, peak, peak_kind, traffic)
     roofline.update({"kernel": "k_step_ct<SetD2V33, N=4> (fused pull-stream + walls + collide)",
                      "bytes_per_launch": bytes_per_launch, "avg_launch_us": avg_launch_s * 1e6})
 
