@@ -73,10 +73,15 @@ def measured_peaks():
     return 6800.0, "fallback"
 
 
-def kernel_source_hash():
+# sources of the step kernel of a precision (fx64.cuh: the fp64 collision only)
+KERNEL_SOURCES = {"fp64": ("k_fp64.cu", "fx64.cuh"), "fp32": ("k_fp32.cu",), "fp16": ("k_fp16.cu",),
+                  "bf16": ("k_bf16.cu",)}
+
+
+def kernel_source_hash(precision):
     h = hashlib.sha256()
     csrc = os.path.join(ROOT, "paper_1510_08886_gb300", "csrc")
-    for fn in ("lbm_kernels.cuh", "lbm_internal.h", "k_fp32.cu", "k_fp64.cu", "fx64.cuh"):
+    for fn in ("lbm_kernels.cuh", "lbm_internal.h") + KERNEL_SOURCES[precision]:
         with open(os.path.join(csrc, fn), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -91,7 +96,7 @@ def ncu_traffic(precision):
     txt = open(path).read()
     m = re.search(r"dram_bytes_per_launch:\s*([0-9.eE+]+)", txt)
     hsh = re.search(r"kernel_source_sha256_16:\s*([0-9a-f]+)", txt)
-    if not m or not hsh or hsh.group(1) != kernel_source_hash():
+    if not m or not hsh or hsh.group(1) != kernel_source_hash(precision):
         return None
     return float(m.group(1))
 
