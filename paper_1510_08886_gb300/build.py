@@ -24,6 +24,9 @@ SOURCES = ["k_fp64.cu", "k_cluster.cu", "k_fp32.cu", "k_fp16.cu", "k_bf16.cu", "
 # sources compiled once more per velocity set, with this macro naming the set
 PER_SET = {"engine_res_fp64.cu": "LBM_RES_SET"}
 SETS = ["SetD2V53", "SetD2V48", "SetD2V40", "SetD2V33", "SetD2V32", "SetD2V16"]
+# (source, macro definition, suffix of the object), the longest first
+UNITS = [(src, f"-D{macro}={s}", "_" + s) for src, macro in PER_SET.items() for s in SETS]
+UNITS += [(src, None, "") for src in SOURCES]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -40,6 +43,11 @@ def _deps():
     return max(os.path.getmtime(f) for f in files)
 
 
+def object_path(unit):
+    src, _, suffix = unit
+    return os.path.join(OUT, os.path.splitext(src)[0] + suffix + ".o")
+
+
 def build(force=False, verbose=False):
     os.makedirs(OUT, exist_ok=True)
     if not force and os.path.exists(LIB) and os.path.getmtime(LIB) >= _deps():
@@ -50,13 +58,9 @@ def build(force=False, verbose=False):
     if verbose:
         common += ["-Xptxas", "-v"]
 
-    # the longest first
-    units = [(src, f"-D{macro}={s}", "_" + s) for src, macro in PER_SET.items() for s in SETS]
-    units += [(src, None, "") for src in SOURCES]
-
     def compile_one(unit):
-        src, define, suffix = unit
-        obj = os.path.join(OUT, os.path.splitext(src)[0] + suffix + ".o")
+        src, define, _ = unit
+        obj = object_path(unit)
         cmd = [nvcc] + common + ([define] if define else []) + ["-c", os.path.join(CSRC, src), "-o", obj]
         if src.endswith(".cpp"):
             cmd = [nvcc, "-O2", "-std=c++17", "-Xcompiler", "-fPIC", "-I", INCLUDE, "-c",
@@ -66,8 +70,8 @@ def build(force=False, verbose=False):
             raise RuntimeError(f"nvcc failed for {src}:\n{r.stdout}\n{r.stderr}")
         return obj, r.stderr
 
-    with cf.ThreadPoolExecutor(max_workers=len(units)) as ex:
-        results = list(ex.map(compile_one, units))
+    with cf.ThreadPoolExecutor(max_workers=len(UNITS)) as ex:
+        results = list(ex.map(compile_one, UNITS))
     if verbose:
         for _, log in results:
             sys.stderr.write(log)

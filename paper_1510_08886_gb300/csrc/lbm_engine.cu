@@ -137,9 +137,12 @@ struct EngSlot {
 
 constexpr size_t kStageBytes = 256 << 10;
 
-// A slot's flags on admission.
-__global__ void k_admit(int* active, unsigned* status) {
-    *active = 1;
+// A slot takes part in the reductions from its admission, the last operation of
+// lbm_engine_add, to its release, which also leaves its status word clear for the
+// next solve.
+__global__ void k_admit(int* active) { *active = 1; }
+__global__ void k_release(int* active, unsigned* status) {
+    *active = 0;
     *status = 0u;
 }
 
@@ -169,7 +172,6 @@ struct lbm_engine {
     lbm::EngineTile* d_tiles = nullptr;
     std::vector<EngSlot> slots;
     std::vector<unsigned char> h_rec;          // host copies of the records
-    std::vector<int> h_active;
     std::vector<double> h_results;
     // asynchronous chunks: per outstanding launch, its results copied in
     // stream order into pinned host memory, and an event marking the copy
@@ -562,10 +564,6 @@ cudaError_t upload_and_init(lbm_engine* e, int slot, double Kn, const double* rh
     const int n = spec.Nx * spec.Ny;
     cudaError_t err = cudaMemcpyAsync(static_cast<char*>(e->d_solves) + size_t(slot) * e->rec_bytes,
                                       &h, sizeof(h), cudaMemcpyHostToDevice, e->stream);
-    if (err == cudaSuccess) {
-        k_admit<<<1, 1, 0, e->stream>>>(e->d_active + slot, h.status);
-        err = cudaGetLastError();
-    }
     // (no density given: the init kernel takes 1 at every node)
     if (err == cudaSuccess && rho_host)
         err = cudaMemcpyAsync(h.prev, rho_host, size_t(n) * 8, cudaMemcpyHostToDevice, e->stream);
@@ -581,6 +579,10 @@ cudaError_t upload_and_init(lbm_engine* e, int slot, double Kn, const double* rh
                       ? lbm::launch_init_fp16(k, spec.N, e->precision == LBM_BF16, rho0, h.f[0], db,
                                               e->stream)
                       : lbm::launch_init_fp32(k, spec.N, rho0, h.f[0], db, e->stream);
+    }
+    if (err == cudaSuccess) {
+        k_admit<<<1, 1, 0, e->stream>>>(e->d_active + slot);
+        err = cudaGetLastError();
     }
     return err;
 }
@@ -659,7 +661,6 @@ int lbm_engine_create(int precision, int max_solves, void* arena, size_t arena_b
     e->d_tiles = reinterpret_cast<lbm::EngineTile*>(e->base + o_tiles);
     e->slots.resize(max_solves);
     e->h_rec.assign(e->rec_bytes * size_t(max_solves), 0);
-    e->h_active.assign(max_solves, 0);
     e->h_results.assign(4 * size_t(max_solves), 0.0);
     const size_t result_bytes = al256(sizeof(double) * 8 * size_t(max_solves));
     if (cudaMallocHost(&e->pinned, result_bytes + kStageBytes) != cudaSuccess) {
@@ -752,9 +753,7 @@ int lbm_engine_add(lbm_engine* e, const lbm_dvm* dvm, int order, int Nx, int Ny,
     sl.g = force;
     cudaError_t err = e->precision == LBM_FP64 ? upload_and_init<double>(e, slot, Kn, rho_host)
                                                : upload_and_init<float>(e, slot, Kn, rho_host);
-    e->h_active[slot] = 1;
     if (err != cudaSuccess) {
-        e->h_active[slot] = 0;
         sl.used = false;
         e->arena.release(off, L.total);
         return cuda_rc(err);
@@ -767,11 +766,10 @@ int lbm_engine_add(lbm_engine* e, const lbm_dvm* dvm, int order, int Nx, int Ny,
 int lbm_engine_remove(lbm_engine* e, int slot) {
     if (!e || slot < 0 || slot >= e->max_slots || !e->slots[slot].used) return LBM_EINVAL;
     EngSlot& sl = e->slots[slot];
-    e->h_active[slot] = 0;
     // stream-ordered: work already queued for this slot finishes before any
     // later use of its memory (a new solve's set-up goes on the same stream)
-    cudaError_t err = cudaMemcpyAsync(e->d_active + slot, &e->h_active[slot], sizeof(int),
-                                      cudaMemcpyHostToDevice, e->stream);
+    k_release<<<1, 1, 0, e->stream>>>(e->d_active + slot, sl.status);
+    const cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return cuda_rc(err);
     e->arena.release(sl.off, sl.bytes);
     sl.used = false;
