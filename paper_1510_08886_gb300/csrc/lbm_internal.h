@@ -28,6 +28,7 @@ constexpr int min_blocks_for(int V, int bytes) {
     const int blocks = 65536 / (regs * kBlock);
     return blocks < 1 ? 1 : (blocks > 16 ? 16 : blocks);
 }
+constexpr int kSMs = 152;            // of a GB300
 constexpr int kReduceBlocks = 304;   // 2 x 152 SMs for the partial sums
 constexpr int kReduceThreads = 256;
 

@@ -35,7 +35,8 @@ namespace lbm {
 // next step's blocks take the slots this step leaves free and compute their
 // indices there; step_wait, before the first access to a lattice or a moment
 // field, returns when every earlier step has completed and its stores are
-// visible.  (Without the launch attribute both do nothing.)  Pointers to a lattice
+// visible.  (Without the launch attribute both do nothing; without step_begin the
+// next step's blocks come as this one's end.)  Pointers to a lattice
 // carry no __restrict__, in the kernels and in their helpers: const __restrict__
 // would allow the read-only load path, whose data are taken to be constant for
 // the whole life of the kernel, and here the last step may still write them.
@@ -1033,6 +1034,21 @@ __host__ __device__ constexpr int step_blocks() {
     return sizeof(C) == 8 ? 5 : min_blocks_for(V, sizeof(C));
 }
 
+// Grid from which a step lets the next one's blocks in before its own have ended:
+// two and a half waves of resident blocks, else they pile up on the SMs that are
+// free first and the next step runs unevenly.  us per step, let in / not: fp64
+// D2V33 1021 x 160 (1.7 waves) 36.9 / 33.0, 1021 x 340 (3.6) 69.8 / 71.8, 4096 x
+// 512 333 / 335; D2V32 1021 x 200 (2.1) 46.9 / 44.9, 1024 x 240 (2.5) 54.1 / 57.3;
+// D2V53 1024 x 240 (3.2) 83.8 / 87.2; fp32 D2V53 2048 x 512 81.5 / 82.9.  The
+// other kernels gain nothing at any size (fp16 D2V33 4096 x 512 63.5 / 63.1, fp64
+// D2V16 4096 x 512 166.9 / 166.5) or lose (fp32 D2V32 1021 x 160 44.9 / 21.5).
+template <class SET, typename C>
+__host__ __device__ constexpr int early_blocks() {
+    constexpr int V = SET::R + 2 * SET::P;
+    constexpr int resident = sizeof(C) == 8 && step_smem<SET, C>() > 45 * 1024 ? 4 : 5;
+    return (sizeof(C) == 8 ? V > 16 : V > 48) ? 5 * resident * kSMs / 2 : 0x7fffffff;
+}
+
 // e_x of plane a of a compiled set (rest, the P pair members, their negatives)
 template <class SET>
 __host__ __device__ constexpr int plane_ex(int a) {
@@ -1158,11 +1174,7 @@ k_step_ct(const __grid_constant__ KParams<C, SET::R + 2 * SET::P> k, const S* sr
     // heavier blocks run first, the uniform interior blocks form the tail);
     // block 2 strips + m then takes the interior block at node (strips + m) 128.
     int blk = int(blockIdx.x);
-    // A grid of several waves lets the next step's blocks into its tail; a small
-    // one lets them in as its blocks end, else they pile up on the SMs that are
-    // free first (fp64 D2V33 257 x 131: 19.6 us per step against 14.7; bf16 D2V40
-    // 320 x 152: 24 against 20)
-    if (gridDim.x >= 8 * 152) step_begin();
+    if (int(gridDim.x) >= early_blocks<SET, C>()) step_begin();
     if (k.strips) {
         if (blk < 2 * k.strips) step_wait();
         if (blk < k.strips) {
@@ -1414,7 +1426,6 @@ k_step_warp(const __grid_constant__ KParams<C, 2 * LP + 1> k, const S* src, S* d
         x = cell - y * k.Nx;
     }
     const bool wb = node && y < k.maxey, wt = node && y >= k.Ny - k.maxey;
-    step_begin();
     step_wait();
     auto ld = [&](int b, int row, int xs) {
         return src[(long long)b * k.plane + (long long)row * k.Nx + xs];
@@ -1466,7 +1477,6 @@ __global__ void __launch_bounds__(kBlock)
 k_generic(const __grid_constant__ KParams<C, MV> k, const S* src,
           const double* __restrict__ rho0, S* dst, const DevBufs b) {
     const int cell = blockIdx.x * kBlock + threadIdx.x;
-    step_begin();
     if (cell >= k.ncell) return;
     const int y = cell / k.Nx;
     const int x = cell - y * k.Nx;

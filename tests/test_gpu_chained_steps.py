@@ -28,9 +28,10 @@ def _solver(name, N, Nx, Ny, precision):
     return s.set_resident(False).init(rho_field(Nx, Ny, seed=29, amplitude=1e-3))
 
 
-# (name, N, Nx, Ny): 1276 and 1280 blocks of 128 nodes, above the 1216 of the
-# early trigger; then 40 blocks, a short column and a small set on lanes
-SHAPES = [("D2V33", 4, 1021, 160), ("D2V33", 4, 1024, 160), ("D3V107xz", 3, 1021, 160),
+# (name, N, Nx, Ny): 2074 and 2080 blocks of 128 nodes, above the 1520 or 1900 from
+# which fp64 and the 53-velocity set let blocks in, and 1276 below; then 40 blocks, a
+# short column and a small set on lanes
+SHAPES = [("D2V33", 4, 1021, 260), ("D2V33", 4, 1024, 260), ("D3V107xz", 3, 1021, 260), ("D2V33", 4, 1021, 160),
           ("D2V16", 3, 129, 39), ("D2V33", 4, 1, 5001), ("D2V16", 3, 1, 40)]
 
 
