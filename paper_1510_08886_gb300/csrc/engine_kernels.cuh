@@ -320,6 +320,27 @@ __device__ __forceinline__ void res_push(const KParams<C, MV>& k, S* sb, int PS,
     }
 }
 
+// dp_node on the populations of node (x, y) where they lie, for either kind of step
+// and any Nx.  One call, apart from the path of the other nodes: in its place the
+// fixed-point collision spills more (D2V33 of 16 to 120 x 3 nodes, 300 channels: 20.3
+// us per step inline, 19.6 as a call).
+template <class SET, int N, int MV>
+__device__ __noinline__ Moments dp_resident(const KParams<double, MV>& k, double* sb, int PS, int x, int y,
+                                            bool step_a, bool tiny) {
+    constexpr int G = set_maxey<SET>();
+    const int Nx = k.Nx, o = (y + G) * Nx + x;
+    // slot that population a of velocity (., ey) is read from; the new value of the
+    // opposite one goes there too
+    auto slot = [&](int a, int opp, int ey) {
+        if (step_a) return a * PS + o;
+        int t = x - k.sx[a];
+        t += t < 0 ? Nx : 0;
+        return opp * PS + (y - ey + G) * Nx + t;
+    };
+    return dp_node<SET, N>(k, tiny, [&](int a, int opp, int, int ey) { return sb[slot(a, opp, ey)]; },
+                           [&](int a, int opp, int, int ey, double v) { sb[slot(opp, a, -ey)] = v; });
+}
+
 // Update of an fp64 node, which reads its populations where they lie: a wall
 // node first writes its wall fills into the slots they would have come from,
 // which only this node touches in this step.
@@ -355,9 +376,11 @@ __device__ __forceinline__ CellCoef<double> res_update64(const KParams<double, M
                     mul_rn(ys < 0 ? pb : pt, k.cw[a]);
         }
     }
-    return collide64<SET, N>(k, want, get, [&](int a, int opp, int ex, int ey, double v) {
-        (STEP_A ? sb[opp * PS + o] : sb[a * PS + at(ex, ey)]) = v;
-    });
+    return collide64<SET, N>(k, want, get,
+                             [&](int a, int opp, int ex, int ey, double v) {
+                                 (STEP_A ? sb[opp * PS + o] : sb[a * PS + at(ex, ey)]) = v;
+                             },
+                             [&](bool tiny) { return dp_resident<SET, N>(k, sb, PS, x, y, STEP_A, tiny); });
 }
 
 template <typename C>

@@ -30,7 +30,7 @@
 //
 // Nodes outside the range of the fixed-point form (a density far from 1, a flow
 // speed near the lattice's limit, non-finite values) and solves whose force
-// constants do not fit take the FP64 evaluation (slow_collide), node by node.
+// constants do not fit take the FP64 evaluation (dp_collide), node by node.
 //
 // The functions are plain C++ with the device's multiply intrinsics spelled out
 // for the host, so that the CPU tests run the same arithmetic.
@@ -278,6 +278,13 @@ struct Sums {
 constexpr int kLeastE = 128, kLargestE = 1021;
 LBM_HD bool exponent_fits(int E) { return E > kLeastE && E <= kLargestE; }
 
+// Bits of the force's constants h and theta, times max |e|, in units U_G at most: the
+// unit of a strong force is set by it, and fewer bits would round coarser than fp64.
+constexpr int kForceRoom = 60;
+// Binary exponent of h and theta below which const_q would shift by more than 63
+// (q >= 1074 + 4 - kLargestE): solves with so small a force take the FP64 form.
+constexpr int kLeastForce = 62 - 63 - (1074 + 4 - kLargestE);
+
 // exponent key of |e| d, lg = log2 of |e|
 LBM_HD unsigned key(double d, int lg) { return (unsigned(dhi(d)) & 0x7fffffffu) + (unsigned(lg) << 20); }
 LBM_HD unsigned umax_(unsigned a, unsigned b) { return a > b ? a : b; }
@@ -325,13 +332,11 @@ LBM_HD int f2i(float x) {
 }
 
 // The per-solve constant mant 2^-exp in the unit 2^-q: integer part and the
-// 32 bits below it, whatever lies below those cut (a force of 2^-33 units of one
-// node's sums is none).
+// 32 bits below it.
 LBM_HD i64 const_q(i64 mant, int exp, int q, unsigned& frac) {
-    int sh = exp - q;                                      // >= 2 (emin)
-    sh = sh < 95 ? sh : 95;
-    frac = unsigned(sh < 32 ? u64(mant) << (32 - sh) : u64(mant) >> (sh - 32));
-    return mant >> (sh < 63 ? sh : 63);
+    const int sh = exp - q;                                // 2 (emin) .. 63 (kLeastForce)
+    frac = unsigned(u64(mant << (64 - sh)) >> 32);
+    return mant >> sh;
 }
 
 constexpr float kGMax = 1.9e9f;      // of the high word of G: |G| < 2^62.9
@@ -367,8 +372,10 @@ LBM_HD bool coefs(const Consts& k, Sums m, int E, Poly& p) {
         bound += rho * k.em * hif(tq);
     }
     bound += k.gm * fm;
-    bool ok = fj < (C2 == 61 ? 5.0e8f : 1.9e9f) && fk < 5.0e8f && 2.0f * fm * un < k.xlim &&
-              delta > -0.4f && delta < 1.9f;
+    // left early: a node out of range pays for the sums only
+    if (!(fj < (C2 == 61 ? 5.0e8f : 1.9e9f) && fk < 5.0e8f && 2.0f * fm * un < k.xlim && delta > -0.4f &&
+          delta < 1.9f && bound < kGMax))
+        return false;
 
     i64 Mx = mulc(shl(m.jx, 63 - C2), k.c2, hfrac);
     const i64 My = mulc(shl(m.jy, 63 - C2), k.c2);
@@ -443,7 +450,7 @@ LBM_HD bool coefs(const Consts& k, Sums m, int E, Poly& p) {
             const i64 axx = mulc(shl(m.kxx, 2), k.k1) - kd + mulc(shl(Hxx, 4 - S2), k.k2_60) + mulc(Mx2, k.k3_62);
             const i64 axy = mulc(shl(m.kxy, 2), k.k1) + mulc(sh_(Sxy, 3 - S2), k.k2_60) + mulc(My2, k.k3h_62);
             const i64 ayy = mulc(shl(m.kyy, 2), k.k1) - kd + mulc(shl(Hyy, 4 - S2), k.k2_60);
-            ok = ok && k.ga * (fabsf_(hif(axx)) + fabsf_(hif(axy)) + fabsf_(hif(ayy))) + bound < kGMax;
+            bound += k.ga * (fabsf_(hif(axx)) + fabsf_(hif(axy)) + fabsf_(hif(ayy)));
             p.d10 -= 3 * axx + ayy;
             p.d01 -= 2 * axy;
             p.d30 += mulc(shl(axx, 64 - C2 + S3), k.c2);
@@ -463,7 +470,7 @@ LBM_HD bool coefs(const Consts& k, Sums m, int E, Poly& p) {
             p.c13 = -p.c13;
         }
     }
-    return ok && bound < kGMax;
+    return bound < kGMax;
 }
 
 // d* = (1 - omega) d + T, T = G omega w already scaled (units 2^(eb - 1084))
@@ -712,8 +719,9 @@ inline Consts make_consts(double c_, double tau_, double dt_, double g_, int R, 
         if (v > 0) {
             mant = i64(ldexpl(frexpl(v, &e), 62));          // v = mant 2^(e - 62)
             // v 2^q < 2^room with q = 1074 + s0 - E
-            const int room = 60 - ilog2_up(emax);
+            const int room = kForceRoom - ilog2_up(emax);
             if (1074 + si.s0 + e - room > k.emin) k.emin = 1074 + si.s0 + e - room;
+            if (e < kLeastForce) k.ok = 0;
         }
         (i ? k.th_m : k.h_m) = mant;
         (i ? k.th_exp : k.h_exp) = 62 - e;
@@ -745,7 +753,7 @@ inline Consts make_consts(double c_, double tau_, double dt_, double g_, int R, 
     k.c2f = float(c * c);
     // M is shifted left by 3 bits with the extra bits, by 2 without, before a product:
     // |M| < 2^60 or 2^61 (a uniform flow's is at most 2^58.8 U_G in the paper's sets)
-    const float room = extra2(emax) ? 2.6e8f : 5.2e8f;
+    const float room = extra2(emax) ? 2.4e8f : 4.8e8f;
     k.gm = em * gj > kGMax / room ? em * gj : kGMax / room;
     k.em = em;
     k.ga = f3 * (4.0f + 4.0f * k.c2f * em * em) * em;

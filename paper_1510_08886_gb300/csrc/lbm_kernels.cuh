@@ -739,7 +739,7 @@ __host__ __device__ constexpr int poly_class(int p) {
 // Deviation units: d* = (1 - omega) d + omega w (Ge +- Go); 16-bit units
 // (coefficients already times omega / S): h* = (1 - omega) h + (Ge +- Go).
 template <class SET, int J, bool HSPACE, typename C, class PARTS, int MV>
-__device__ __forceinline__ void poly_pair(const KParams<C, MV>& k, const PARTS& pp, C* f) {
+__device__ __forceinline__ void poly_pair(const KParams<C, MV>& k, const PARTS& pp, C& fp, C& fm) {
     constexpr int EX = SET::ex[J], EY = SET::ey[J];
     constexpr bool nx = EX < 0, ny = EY < 0;
     const C Ge = (nx != ny) ? pp.Ee - pp.Eo : pp.Ee + pp.Eo;
@@ -747,8 +747,6 @@ __device__ __forceinline__ void poly_pair(const KParams<C, MV>& k, const PARTS& 
     if constexpr (EX == 0) Go = ny ? -pp.Oy : pp.Oy;
     else if constexpr (EY == 0) Go = nx ? -pp.Ox : pp.Ox;
     else Go = nx ? (ny ? -(pp.Ox + pp.Oy) : pp.Oy - pp.Ox) : (ny ? pp.Ox - pp.Oy : pp.Ox + pp.Oy);
-    C& fp = f[SET::R + J];
-    C& fm = f[SET::R + SET::P + J];
     const C omo = k.one_m_omega;
     if constexpr (HSPACE) {
         fp = fma(omo, fp, Ge + Go);
@@ -766,7 +764,8 @@ __device__ __forceinline__ void poly_class_relax(const KParams<C, MV>& k, const 
                                                  std::integer_sequence<int, J...>) {
     if constexpr (poly_class<SET>(P0) == P0) {
         const PolyParts<iabs(SET::ex[P0]), iabs(SET::ey[P0]), N, C> pp(pc);
-        ((poly_class<SET>(J) == P0 ? poly_pair<SET, J, HSPACE, C>(k, pp, f) : void()), ...);
+        ((poly_class<SET>(J) == P0 ? poly_pair<SET, J, HSPACE, C>(k, pp, f[SET::R + J], f[SET::R + SET::P + J])
+                                   : void()), ...);
     }
 }
 
@@ -829,35 +828,59 @@ __device__ __forceinline__ void relax_ct(const KParams<C, MV>& k, const CellCoef
     }
 }
 
-// FP64 collision of one node with run-time loops over the pairs: what a node
-// outside the range of the fixed-point form takes.
-template <int N, class GET, class PUT, int MV>
-__device__ __forceinline__ CellCoef<double> slow_collide(const KParams<double, MV>& k, const GET& get,
-                                                         const PUT& put) {
-    const int R = k.R, P = k.P;
-    double drho = R ? get(0, 0, 0, 0) : 0.0, Jx = 0, Jy = 0, Kxx = 0, Kxy = 0, Kyy = 0;
-#pragma unroll 1
-    for (int p = 0; p < P; ++p) {
-        const int a = R + p, b = R + P + p, x = k.ex[a], y = k.ey[a];
-        const double fp = get(a, b, x, y), fm = get(b, a, -x, -y);
-        const double sum = fp + fm, dif = fp - fm;
-        drho += sum;
-        Jx = fma(k.pex[p], dif, Jx);
-        Jy = fma(k.pey[p], dif, Jy);
-        Kxx = fma(k.pexx[p], sum, Kxx);
-        Kxy = fma(k.pexy2[p], sum, Kxy);
-        Kyy = fma(k.peyy[p], sum, Kyy);
+// FP64 collision of one node, its populations read where they lie (get, put: see
+// fx::collide): what a solve or a node outside the range of the fixed-point form
+// takes.  Unrolled with the set's numbers like relax_ct, so that it issues no more
+// FP64 operations than the values in registers would need; the FP64 pipe bounds
+// it, and what the node spent on the fixed-point form before it was found out of
+// range runs beside it on the integer pipes.
+template <class SET, int J, int N, class PARTS, class GET, class PUT, int MV>
+__device__ __forceinline__ void dp_poly_pair(const KParams<double, MV>& k, const PARTS& pp, const GET& get,
+                                             const PUT& put) {
+    constexpr int a = SET::R + J, b = SET::R + SET::P + J, x = SET::ex[J], y = SET::ey[J];
+    double fp = get(a, b, x, y), fm = get(b, a, -x, -y);
+    poly_pair<SET, J, false, double>(k, pp, fp, fm);
+    put(a, b, x, y, fp);
+    put(b, a, -x, -y, fm);
+}
+template <class SET, int P0, int N, class GET, class PUT, int MV, int... J>
+__device__ __forceinline__ void dp_poly_class(const KParams<double, MV>& k, const PolyCoef<double>& pc,
+                                              const GET& get, const PUT& put, std::integer_sequence<int, J...>) {
+    if constexpr (poly_class<SET>(P0) == P0) {
+        const PolyParts<iabs(SET::ex[P0]), iabs(SET::ey[P0]), N, double> pp(pc);
+        ((poly_class<SET>(J) == P0 ? dp_poly_pair<SET, J, N>(k, pp, get, put) : void()), ...);
     }
-    const CellCoef<double> q = cell_coef<N, double>(k, drho, Jx, Jy, Kxx, 0.5 * Kxy, Kyy);
-    if (R) put(0, 0, 0, 0, fma(k.one_m_omega, get(0, 0, 0, 0), k.omw_rest * q.a0));
-#pragma unroll 1
-    for (int p = 0; p < P; ++p) {
-        const int a = R + p, b = R + P + p, x = k.ex[a], y = k.ey[a];
-        double fp = get(a, b, x, y), fm = get(b, a, -x, -y);
-        if (k.force) pair_update<true, double>(k, q, p, fp, fm);
-        else pair_update<false, double>(k, q, p, fp, fm);
-        put(a, b, x, y, fp);
-        put(b, a, -x, -y, fm);
+}
+template <class SET, int J, int N, class GET, class PUT, int MV>
+__device__ __forceinline__ void dp_free_pair(const KParams<double, MV>& k, const CellCoef<double>& q, const GET& get,
+                                             const PUT& put) {
+    constexpr int a = SET::R + J, b = SET::R + SET::P + J, x = SET::ex[J], y = SET::ey[J];
+    double fp = get(a, b, x, y), fm = get(b, a, -x, -y);
+    pair_update_free<x, y, N, false, double>(q, k.pomw[J], k.one_m_omega, 1.0, fp, fm);
+    put(a, b, x, y, fp);
+    put(b, a, -x, -y, fm);
+}
+template <class SET, int J, class GET>
+__device__ __forceinline__ void dp_moment_pair(const GET& get, double& drho, double& Jx, double& Jy, double& Kxx,
+                                               double& Kxy, double& Kyy) {
+    constexpr int a = SET::R + J, b = SET::R + SET::P + J, x = SET::ex[J], y = SET::ey[J];
+    moment_pair<x, y, double>(get(a, b, x, y), get(b, a, -x, -y), drho, Jx, Jy, Kxx, Kxy, Kyy);
+}
+template <class SET, int N, class GET, class PUT, int MV, int... I>
+__device__ __forceinline__ CellCoef<double> dp_collide(const KParams<double, MV>& k, const GET& get, const PUT& put,
+                                                       std::integer_sequence<int, I...> pairs) {
+    constexpr int R = SET::R;
+    double drho = 0.0, Jx = 0, Jy = 0, Kxx = 0, Kxy = 0, Kyy = 0;
+    if constexpr (R != 0) drho = get(0, 0, 0, 0);
+    (dp_moment_pair<SET, I>(get, drho, Jx, Jy, Kxx, Kxy, Kyy), ...);
+    const CellCoef<double> q = cell_coef<N, double>(k, drho, Jx, Jy, Kxx, Kxy, Kyy);
+    fx::phase();
+    if constexpr (R != 0) put(0, 0, 0, 0, fma(k.one_m_omega, get(0, 0, 0, 0), k.omw_rest * q.a0));
+    if (k.force) {
+        const PolyCoef<double> pc = poly_coef<N, true, false, double>(q, 1.0);
+        (dp_poly_class<SET, I, N>(k, pc, get, put, pairs), ...);
+    } else {
+        (dp_free_pair<SET, I, N>(k, q, get, put), ...);
     }
     return q;
 }
@@ -886,21 +909,55 @@ __device__ __forceinline__ void fx_moments(const KParams<double, MV>& k, const f
     q.uy = fma(mul_rn(k.c, val(m.jy)), inv, k.hdt_gy);
 }
 
+// A node whose populations are all zero, without a force: they stay zero.  False,
+// nothing put, if one is not.
+template <class GET, class PUT, int MV>
+__device__ __forceinline__ bool keep_rest(const KParams<double, MV>& k, const GET& get, const PUT& put) {
+    auto opp = [&](int a) { return a < k.R ? a : (a < k.R + k.P ? a + k.P : a - k.P); };
+#pragma unroll 1
+    for (int a = 0; a < k.V; ++a)
+        if (get(a, opp(a), k.ex[a], k.ey[a]) != 0.0) return false;
+#pragma unroll 1
+    for (int a = 0; a < k.V; ++a) put(a, opp(a), k.ex[a], k.ey[a], 0.0);
+    return true;
+}
+
+// rho - 1 and u of a node.
+struct Moments {
+    double drho, ux, uy;
+};
+
+// A node outside the fixed-point range (tiny: its populations are below it).
+template <class SET, int N, class GET, class PUT, int MV>
+__device__ __forceinline__ Moments dp_node(const KParams<double, MV>& k, bool tiny, const GET& get, const PUT& put) {
+    if (tiny && !k.force && keep_rest(k, get, put)) return Moments{0.0, 0.0, 0.0};
+    const CellCoef<double> q = dp_collide<SET, N>(k, get, put, std::make_integer_sequence<int, SET::P>{});
+    return Moments{q.drho, q.ux, q.uy};
+}
+
 // fp64 collision of a node of a compiled set (get, put: see fx::collide).  The
 // moments rho, u of the result are valid when want is set; drho and rho are
-// always fit for flag_density.
-template <class SET, int N, class GET, class PUT, int MV>
+// always fit for flag_density.  outside(tiny) does dp_node for a node that the
+// fixed-point form leaves.
+template <class SET, int N, class GET, class PUT, class OUTSIDE, int MV>
 __device__ __forceinline__ CellCoef<double> collide64(const KParams<double, MV>& k, bool want, const GET& get,
-                                                      const PUT& put) {
+                                                      const PUT& put, const OUTSIDE& outside) {
     fx::Sums m;
-    int E;
+    int E = fx::kLargestE + 1;
     const bool done = k.force ? fx::collide<SET, N, true>(k.fx, k.one_m_omega, m, E, get, put)
                               : fx::collide<SET, N, false>(k.fx, k.one_m_omega, m, E, get, put);
-    if (!done) return slow_collide<N>(k, get, put);
     CellCoef<double> q;
     q.drho = 0.0;
     q.rho = 1.0;
-    if (want) fx_moments<fx::guard_bits<SET>()>(k, m, E, q);
+    if (!done) {
+        const Moments d = outside(E <= fx::kLeastE);
+        q.drho = d.drho;
+        q.rho = 1.0 + d.drho;
+        q.ux = d.ux;
+        q.uy = d.uy;
+    } else if (want) {
+        fx_moments<fx::guard_bits<SET>()>(k, m, E, q);
+    }
     return q;
 }
 
@@ -1007,8 +1064,9 @@ __device__ __forceinline__ CellCoef<C> finish_node(const KParams<C, MV>& k, C* f
     if constexpr (sizeof(C) == 8) {
         const double* sf = step_scratch();
         copies_done();
-        return collide64<SET, N>(k, want, [&](int a, int, int, int) { return sf[a * kBlock]; },
-                                 [&](int a, int, int, int, double v) { put(a, v); });
+        auto get = [&](int a, int, int, int) { return sf[a * kBlock]; };
+        auto out = [&](int a, int, int, int, double v) { put(a, v); };
+        return collide64<SET, N>(k, want, get, out, [&](bool tiny) { return dp_node<SET, N>(k, tiny, get, out); });
     } else {
         const CellCoef<C> q = relax_node<SET, N, S, C>(k, f);
         if constexpr (put_as_packed<SET, S>()) {
@@ -1384,7 +1442,7 @@ __device__ __forceinline__ CellCoef<double> warp_node_fx(const KParams<double, M
     node_sum6<LP, long long>(m, p);
     const fx::Sums s{m[0], m[1], m[2], m[3], m[4], m[5]};
     fx::Poly c;
-    ok = fx::exponent_fits(E) && fx::coefs<FMT, N, FORCE>(k.fx, s, Es, c);
+    ok = !node || (fx::exponent_fits(E) && fx::coefs<FMT, N, FORCE>(k.fx, s, Es, c));
     if (!ok || !node) return q;
     const int eb = Es + 10 + 64 - S0;
     if (act) {
@@ -1426,6 +1484,20 @@ __device__ __forceinline__ CellCoef<C> warp_node_any(const KParams<C, MV>& k, in
                 else go(fx::FamilyFormat<2>{});
             } else {
                 go(fx::FamilyFormat<1>{});
+            }
+            if (__all_sync(0xffffffffu, ok)) return q;
+            // a node of zero populations without a force keeps them
+            constexpr unsigned all = LP == 32 ? 0xffffffffu : (1u << LP) - 1u;
+            const unsigned zero = __ballot_sync(0xffffffffu, fp == C(0) && fm == C(0) && f0 == C(0));
+            const bool rest = !k.force && ((zero >> ((threadIdx.x & 31) - p)) & all) == all;
+            if (!ok && rest) {
+                if (p < k.P) {
+                    put(k.R + p, C(0));
+                    put(k.R + k.P + p, C(0));
+                }
+                if (p == 0 && k.R) put(0, C(0));
+                q.rho = C(1);
+                ok = true;
             }
             if (__all_sync(0xffffffffu, ok)) return q;
             const CellCoef<C> r = warp_node<LP, N, C>(k, p, node, pc, fp, fm, f0, [&](int a, C v) {
