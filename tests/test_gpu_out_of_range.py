@@ -122,3 +122,27 @@ def test_rest_stays_at_rest(name, N, Nx, Ny):
     reach = 2 * int(np.max(np.abs(e)))
     if Ny // 2 - reach > 0:
         assert not np.any(s.moments()[1][:Ny // 2 - reach])
+
+
+# channels of more than eight warps per CTA, on 8, 16 and 32 lanes per node
+LARGE = [("D2V16", 3, 1, 600), ("D2V16", 3, 1, 1500), ("D2V16", 3, 5, 290), ("D2V33", 4, 1, 400), ("D3V107xz", 3, 1, 200),
+         ("D3V112xz", 3, 2, 150)]
+
+
+@pytest.mark.parametrize("precision,amplitude", [("fp32", 1e-3), ("fp64", 1e-3), ("fp64", 0.3)])
+@pytest.mark.parametrize("name,N,Nx,Ny", LARGE)
+def test_large_cluster_blocks_bitwise_equal_launched(name, N, Nx, Ny, precision, amplitude):
+    """Resident steps give the bits of launched steps; with the larger density
+    amplitude nodes of one warp split between the fixed-point and the FP64 form."""
+    import paper_1510_08886_gb300 as lbm
+    e, w, c = lbm.dvm(name)
+    rho = np.clip(rho_field(Nx, Ny, seed=5, amplitude=amplitude), 0.2, None)
+    g = oracle.force_for_mach(0.2, 1e-2)
+    a, b = (lbm.Solver(e, w, c, N, Nx, Ny, 0.2, g, precision=precision).set_resident(r).init(rho) for r in (True, False))
+    assert a.resident_ctas() > 0 and b.resident_ctas() == 0
+    for n in (2, 1, 30):
+        a.step(n)
+        b.step(n)
+        assert np.array_equal(a.populations(), b.populations())
+        for x, y in zip(a.moments(), b.moments()):
+            assert np.array_equal(x, y)
