@@ -14,8 +14,9 @@
 // Bound by one node's dependency chain: in fp64 ~700 integer instructions for the
 // coefficients on every lane, the sums over the lanes and the cluster barrier
 // (~370 cycles).  D2V16 1 x 64: 2.6 us per step (4.3 when ~100 FP64 instructions
-// of 64 cycles each made the chain); 1 x 1500, 24 warps per CTA: 6.3 us against
-// 9.2 with one launch per step (fp32: 2.0 against 8.3).
+// of 64 cycles each made the chain); 1 x 600, 10 warps per CTA: 4.1 us against 6.0
+// with one launch per step; 1 x 1500, 24 warps: 6.7 against 6.0 (fp32: 2.2 against
+// 5.3).
 //
 // No thread leaves before the last barrier: every thread executes the same K + 1
 // cluster barriers, so the barrier cannot wait on a CTA that has exited, and no
@@ -174,8 +175,10 @@ k_chunk_cluster(const __grid_constant__ KParams<C, 2 * LP + 1> k, const S* fin, 
         const C fm = act ? value(sm, pb, pt, to, k.R + k.P + p) : C(0);
         const C f0 = has0 ? value(s0, pb, pt, to, 0) : C(0);
         auto put = [&](int a, C v) { dst[a * lplane + cl] = S(v); };
-        const CellCoef<C> q = warp_node_any<LP, N, C>(k, p, node, pc, pf, fp, fm, f0, s >= K - 2, put);
+        bool left;
+        const CellCoef<C> q = warp_node_any<LP, N, C>(k, p, node, pc, pf, fp, fm, f0, s >= K - 2, left, put);
         if (node && p == 0) {
+            if (MAXT > kClusterThreadsDp && left && s == K - 1) atomicOr(b.status, kStatusLeftRange);
             if (s == K - 1) store_moments<C>(q, int(g0 + cl), b);
             else if (emit_prev && s == K - 2) b.prev_ux[g0 + cl] = (double)q.ux;
             flag_density<C>(q, b.status);
@@ -210,12 +213,12 @@ void* pick_sized(int N, int LP) {
     }
 }
 
-// 256-thread blocks may use all the registers they want; more rows per CTA than
-// that need the larger block's 80 (fp32 D2V33 3 x 80 with those: 2.91 us per step
-// against 2.48, D2V16 5 x 29 1.86 against 1.72).
+// Blocks of kClusterThreadsDp threads may use all the registers they want; more
+// rows per CTA than that need the larger block's 80 (fp32 D2V33 3 x 80 with those:
+// 2.91 us per step against 2.48, D2V16 5 x 29 1.86 against 1.72).
 template <typename C>
 void* pick_kernel(int N, int LP, int threads) {
-    return threads <= 256 ? pick_sized<256, C>(N, LP) : pick_sized<kClusterThreads, C>(N, LP);
+    return threads <= kClusterThreadsDp ? pick_sized<kClusterThreadsDp, C>(N, LP) : pick_sized<kClusterThreads, C>(N, LP);
 }
 
 cudaLaunchConfig_t cluster_config(const ClusterPlan& pl, cudaStream_t st, cudaLaunchAttribute* at) {
@@ -243,6 +246,9 @@ cudaLaunchConfig_t cluster_config(const ClusterPlan& pl, cudaStream_t st, cudaLa
 template <typename C>
 int plan_cluster_t(const KParams<C>& k, int N, int LP, ClusterPlan& pl) {
     pl = ClusterPlan{};
+    int max_threads = kClusterThreads;
+    if constexpr (sizeof(C) == 8)
+        if (!(k.fx.ok && fx_lanes(LP, k.fx.fam))) max_threads = kClusterThreadsDp;
     int dev = 0, optin = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
@@ -259,7 +265,7 @@ int plan_cluster_t(const KParams<C>& k, int N, int LP, ClusterPlan& pl) {
         const int rows = (k.Ny + cmax - 1) / cmax;
         const int ctas = (k.Ny + rows - 1) / rows;
         const int groups = (rows * k.Nx + G - 1) / G;      // warps of work per CTA
-        if (groups > kClusterThreads / 32) continue;
+        if (groups > max_threads / 32) continue;
         void* fn = pick_kernel<C>(N, LP, 32 * groups);
         if (!fn) return 0;
         const size_t need = ((size_t(2) * k.V * rows * k.Nx * sizeof(C) + 15) & ~size_t(15)) +

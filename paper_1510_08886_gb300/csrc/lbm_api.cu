@@ -34,6 +34,7 @@ struct lbm_solver : lbm::SolveSpec {
     // tiny fp64 / fp32 channels: chunks of steps resident on one thread-block cluster
     lbm::ClusterPlan cl{};
     bool resident = true;
+    bool left_range = false;         // seen in the status: see kClusterThreadsDp
     std::vector<char> readback;      // lbm_moments of a small channel
 };
 
@@ -424,9 +425,23 @@ int launch_step(lbm_solver* s, int emit) {
     return LBM_OK;
 }
 
+void drop_graphs(lbm_solver* s) {
+    for (int i = 0; i < 2; ++i) {
+        if (s->chunk_exec[i]) cudaGraphExecDestroy(s->chunk_exec[i]);
+        s->chunk_exec[i] = nullptr;
+        s->chunk_K[i] = 0;
+    }
+}
+
+void set_left_range(lbm_solver* s, bool v) {
+    if (s->left_range != v) drop_graphs(s);
+    s->left_range = v;
+}
+
 int launch_init(lbm_solver* s, const double* rho_dev) {
     s->cur = 0;
     s->steps = 0;
+    set_left_range(s, false);
     cudaError_t e = cudaMemsetAsync(s->b.status, 0, sizeof(unsigned), s->stream);
     if (e != cudaSuccess) return cuda_status(e);
     if (is16(s->precision) && s->scale != 1.0 / 64.0) {
@@ -448,6 +463,12 @@ int launch_init(lbm_solver* s, const double* rho_dev) {
     return cuda_status(e);
 }
 
+// What a status word read from the device means for the caller.
+int take_status(lbm_solver* s, unsigned st) {
+    if (st & lbm::kStatusLeftRange) set_left_range(s, true);
+    return st & lbm::kStatusDensity ? LBM_ENONFINITE : LBM_OK;
+}
+
 // The four reduction results and the status word, which follows them in the
 // workspace, in one copy: an error of the copy, else the solve's status.
 int read_results(lbm_solver* s, double out[4]) {
@@ -459,7 +480,7 @@ int read_results(lbm_solver* s, double out[4]) {
     std::memcpy(out, host, 4 * sizeof(double));
     unsigned st = 0;
     std::memcpy(&st, host + kResultsToStatus, sizeof(st));
-    return st ? LBM_ENONFINITE : LBM_OK;
+    return take_status(s, st);
 }
 
 int reduce(lbm_solver* s, bool with_prev, double out[4]) {
@@ -477,7 +498,7 @@ int read_status(lbm_solver* s) {
     cudaError_t e = cudaMemcpyAsync(&st, s->b.status, sizeof(st), cudaMemcpyDeviceToHost, s->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
     if (e != cudaSuccess) return cuda_status(e);
-    return st ? LBM_ENONFINITE : LBM_OK;
+    return take_status(s, st);
 }
 
 // 16-bit storage: make max |h| over the state lie in (1/2, 1] by a power-of-2
@@ -504,7 +525,7 @@ int refresh_scale(lbm_solver* s) {
 }
 
 bool resident_on(const lbm_solver* s) {
-    return s->resident && s->cl.ctas > 0 &&
+    return s->resident && s->cl.ctas > 0 && !s->left_range &&
            (s->precision == LBM_FP64 || s->precision == LBM_FP32);
 }
 
@@ -815,13 +836,7 @@ int lbm_run_to_steady(lbm_solver* s, double tol, long max_steps, long check_ever
 
 int lbm_set_resident(lbm_solver* s, int enable) {
     if (!s || (enable != 0 && enable != 1)) return LBM_EINVAL;
-    if (s->resident != bool(enable)) {
-        for (int i = 0; i < 2; ++i) {
-            if (s->chunk_exec[i]) cudaGraphExecDestroy(s->chunk_exec[i]);
-            s->chunk_exec[i] = nullptr;
-            s->chunk_K[i] = 0;
-        }
-    }
+    if (s->resident != bool(enable)) drop_graphs(s);
     s->resident = bool(enable);
     return LBM_OK;
 }
@@ -855,7 +870,7 @@ int lbm_moments(lbm_solver* s, double* rho, double* ux, double* uy) {
         std::memcpy(uy, h + (reinterpret_cast<char*>(s->b.uy) - first), n);
         unsigned st = 0;
         std::memcpy(&st, h + span - sizeof(st), sizeof(st));
-        return st ? LBM_ENONFINITE : LBM_OK;
+        return take_status(s, st);
     }
     if (rho && e == cudaSuccess) e = cudaMemcpyAsync(rho, s->b.rho, n, cudaMemcpyDeviceToHost, s->stream);
     if (ux && e == cudaSuccess) e = cudaMemcpyAsync(ux, s->b.ux, n, cudaMemcpyDeviceToHost, s->stream);
@@ -979,6 +994,7 @@ int lbm_set_state(lbm_solver* s, const void* host, size_t bytes) {
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
     if (e != cudaSuccess) return cuda_status(e);
     s->steps = h.steps;
+    set_left_range(s, false);
     if (is16(s->precision)) {
         s->scale = h.scale;
         lbm::fill_params(*s, s->k32);

@@ -153,6 +153,10 @@ inline KParams<C, MV> shrink_params(const KParams<C>& k) {
     return d;
 }
 
+// Status word of a solve: a density that is not positive and finite was seen;
+// nodes of a large resident block were outside the fixed-point range.
+constexpr unsigned kStatusDensity = 1u, kStatusLeftRange = 2u;
+
 // Device buffers of one solver.
 struct DevBufs {
     void* f[2];                  // population lattices (ping-pong)
@@ -200,7 +204,12 @@ inline int warp_path_lanes(int P, long long ncell) {
 // Resident chunks of a tiny fp64 or fp32 channel on one thread-block cluster
 // (k_cluster.cu): CTAs of at most kClusterThreads threads, shared memory padded
 // to kClusterSmemPad (more than half an SM's) so that no two share an SM.
-constexpr int kClusterThreads = 768;
+// fp64 nodes on the FP64 pipe (two lanes per SM) run faster on all SMs with a launch
+// per step than more than kClusterThreadsDp / 32 warps of them on each SM of a cluster
+// (D2V16 1 x 1500: 7.6 us per step against 23.2): solves outside the fixed-point
+// range have no larger block, and a channel whose nodes leave it sets
+// kStatusLeftRange, which the host heeds where it reads the status.
+constexpr int kClusterThreads = 768, kClusterThreadsDp = 256;
 constexpr int kClusterSmemPad = 116 * 1024;
 constexpr long kClusterMaxK = 4096;           // steps per launch in lbm_step
 struct ClusterPlan {

@@ -462,7 +462,7 @@ __device__ __forceinline__ void flag_density(const CellCoef<C>& q, unsigned int*
         const int bits = __float_as_int(q.rho);
         ok = bits > 0 && bits < 0x7f800000;
     }
-    if (!ok) atomicOr(status, 1u);
+    if (!ok) atomicOr(status, kStatusDensity);
 }
 
 template <typename C>
@@ -1460,16 +1460,21 @@ __device__ __forceinline__ CellCoef<double> warp_node_fx(const KParams<double, M
     return q;
 }
 
+// Pairs of LP lanes whose fixed-point form the kernels know (SetInfo::fam).
+__host__ __device__ constexpr bool fx_lanes(int LP, int fam) {
+    return LP == 8 ? fam == 0 : (LP == 16 ? fam == 0 || fam == 2 : fam == 1);
+}
+
 // warp_node, in fixed point where it applies.  A node outside its range takes
-// the FP64 form, with the whole warp in step (the forms shuffle).
+// the FP64 form, with the whole warp in step (the forms shuffle); left: it did,
+// in a solve that could have had the fixed-point form.
 template <int LP, int N, typename C, class PUT, int MV>
 __device__ __forceinline__ CellCoef<C> warp_node_any(const KParams<C, MV>& k, int p, bool node,
                                                      const PairConst<C>& pc, const PairFx& pf, C fp, C fm, C f0,
-                                                     bool want, const PUT& put) {
+                                                     bool want, bool& left, const PUT& put) {
+    left = false;
     if constexpr (sizeof(C) == 8) {
-        // (the compiled sets of P <= 8, 16 and 32 pairs are of these families)
-        const bool fits = LP == 8 ? k.fx.fam == 0 : (LP == 16 ? k.fx.fam == 0 || k.fx.fam == 2 : k.fx.fam == 1);
-        if (k.fx.ok && fits) {
+        if (k.fx.ok && fx_lanes(LP, k.fx.fam)) {
             bool ok = false;
             CellCoef<C> q{};
             auto go = [&](auto fmt) {
@@ -1500,6 +1505,7 @@ __device__ __forceinline__ CellCoef<C> warp_node_any(const KParams<C, MV>& k, in
                 ok = true;
             }
             if (__all_sync(0xffffffffu, ok)) return q;
+            left = !ok;
             const CellCoef<C> r = warp_node<LP, N, C>(k, p, node, pc, fp, fm, f0, [&](int a, C v) {
                 if (!ok) put(a, v);
             });
@@ -1550,8 +1556,9 @@ k_step_warp(const __grid_constant__ KParams<C, 2 * LP + 1> k, const S* src, S* d
     const C f0 = (node && p == 0 && k.R) ? value(0) : C(0);
     unsigned rs = sr_seed<S, C>(k.seed, cell);
     auto put = [&](int a, C v) { dst[(long long)a * k.plane + cell] = st_pop<S, C>(k, v, a, rs); };
+    bool left;
     const CellCoef<C> q = warp_node_any<LP, N, C>(k, p, node, pc, pair_fx(k, act ? p : 0), fp, fm, f0,
-                                                  k.emit != 0, put);
+                                                  k.emit != 0, left, put);
     if (node && p == 0) {
         emit_moments<C>(k, q, cell, b);
         flag_density<C>(q, b.status);

@@ -133,16 +133,37 @@ LARGE = [("D2V16", 3, 1, 600), ("D2V16", 3, 1, 1500), ("D2V16", 3, 5, 290), ("D2
 @pytest.mark.parametrize("name,N,Nx,Ny", LARGE)
 def test_large_cluster_blocks_bitwise_equal_launched(name, N, Nx, Ny, precision, amplitude):
     """Resident steps give the bits of launched steps; with the larger density
-    amplitude nodes of one warp split between the fixed-point and the FP64 form."""
+    amplitude nodes of one warp split between the fixed-point and the FP64 form,
+    and once the host has read the status the solve goes on in launches."""
     import paper_1510_08886_gb300 as lbm
     e, w, c = lbm.dvm(name)
     rho = np.clip(rho_field(Nx, Ny, seed=5, amplitude=amplitude), 0.2, None)
     g = oracle.force_for_mach(0.2, 1e-2)
     a, b = (lbm.Solver(e, w, c, N, Nx, Ny, 0.2, g, precision=precision).set_resident(r).init(rho) for r in (True, False))
     assert a.resident_ctas() > 0 and b.resident_ctas() == 0
-    for n in (2, 1, 30):
+    for n in (33, 2, 1):
         a.step(n)
         b.step(n)
         assert np.array_equal(a.populations(), b.populations())
         for x, y in zip(a.moments(), b.moments()):
             assert np.array_equal(x, y)
+    a.init(rho)
+    assert a.resident_ctas() > 0
+    if amplitude > 0.1:
+        a.step(2)                       # density well out of range at some nodes
+        assert a.status() == 0 and a.resident_ctas() == 0
+        b.init(rho).step(2)
+        assert a.run_to_steady(1e-16, 203, check_every=50) == b.run_to_steady(1e-16, 203, check_every=50)
+        assert np.array_equal(a.populations(), b.populations())
+        a.set_state(b.get_state())
+        assert a.resident_ctas() > 0
+
+
+def test_fixed_point_clusters_only():
+    """A solve outside the range as a whole gets no block of more than eight warps
+    (two FP64 lanes per SM), one inside does."""
+    import paper_1510_08886_gb300 as lbm
+    e, w, c, Kn, g = _case("D2V16", "theta", 1500)
+    assert lbm.Solver(e, w, c, 3, 1, 1500, Kn, g).resident_ctas() == 0
+    assert lbm.Solver(e, w, c, 3, 1, 64, Kn, g).resident_ctas() > 0
+    assert lbm.Solver(e, w, c, 3, 1, 1500, 0.1, 1e-3).resident_ctas() > 0
