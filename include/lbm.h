@@ -51,7 +51,14 @@ enum {
 
 /* Storage precision of the populations.  Every precision stores the
  * deviation d_a = fbar_a - w_a from the rest state at rho0 = 1.
- *   LBM_FP64: d in fp64, fp64 arithmetic;
+ *   LBM_FP64: d in fp64.  The collision of a velocity set with compiled kernels
+ *     (see lbm_engine) runs in 64-bit fixed point with one exponent per node,
+ *     the error of a node's density and momentum 0.2 to 1.2 times that of fp64
+ *     arithmetic, for solves with
+ *     tau c |g| < 1/8, |g| = 0 or c |g| min(tau, dt/2) >= 2^-59 and weights of
+ *     (e_x, e_y) and (-e_x, e_y) equal to 1e-15, at nodes with 0.6 < rho < 2.9
+ *     and c (|u_x| + |u_y|) max|e_a| < 0.4; other solves and nodes, and other
+ *     velocity sets, in fp64 arithmetic, several times slower;
  *   LBM_FP32: d in fp32, fp32 arithmetic;
  *   LBM_FP16, LBM_BF16: h_a = d_a / (w_a S) in IEEE half / bfloat16, fp32
  *     arithmetic; S is a per-solve power of 2 (initially 2^-6) that
@@ -186,11 +193,15 @@ int lbm_step(lbm_solver* s, long nsteps);
 /* Resident chunks for tiny fp64 and fp32 channels (no counterpart in the
  * paper, which does not discuss execution).  A channel whose step runs on
  * several lanes per node (at most 152*32*8 node-lanes) and whose rows fit one
- * thread-block cluster (at most 16 CTAs of at most 8 warps, both lattices in
- * their shared memory) runs many steps per launch, the cluster's barrier
+ * thread-block cluster (at most 16 CTAs of at most 24 warps, 8 for an fp64 solve
+ * outside the fixed-point range of LBM_FP64; both lattices in their shared
+ * memory) runs many steps per launch, the cluster's barrier
  * between steps, instead of one launch per step; lbm_step and
  * lbm_run_to_steady then use it.  The result is bitwise that of the per-step
- * launches.  enable: 1 (the default at lbm_create) or 0; anything else ->
+ * launches.  (An fp64 channel of more than 8 warps per CTA whose nodes leave the
+ * fixed-point range goes on with single launches, which are faster for them,
+ * from the next call that reads its status until it is initialised again.)
+ * enable: 1 (the default at lbm_create) or 0; anything else ->
  * LBM_EINVAL.  16-bit storage and larger channels ignore the setting. */
 int lbm_set_resident(lbm_solver* s, int enable);
 
@@ -276,7 +287,7 @@ int lbm_set_state(lbm_solver* s, const void* host, size_t bytes);
  * is admitted only if its footprint (lbm_engine_solve_bytes) fits.
  * Supported: the velocity sets with compiled kernels (the paper's D2V16,
  * D2V32, D2V33 and the (x, z) marginals of D3V107, D3V96, D3V112;
- * LBM_ENOTSUP otherwise), storage LBM_FP64 (fp64 arithmetic), LBM_FP32,
+ * LBM_ENOTSUP otherwise), storage LBM_FP64, LBM_FP32,
  * LBM_FP16 or LBM_BF16 (fp32 arithmetic; the 16-bit scale S stays 2^-6 in the
  * engine).  Each solve's arithmetic is the one of lbm_step's compiled-set
  * kernel, so a solve's results do not depend on which other solves share the

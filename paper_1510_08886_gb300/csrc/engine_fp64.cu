@@ -1,4 +1,4 @@
-// Engine kernels with fp64 population storage and fp64 arithmetic: the
+// Engine kernels with fp64 population storage (collision: fx64.cuh): the
 // per-step tiled kernel, its occupancy, and the per-slot reductions of fp64
 // slot records.
 #include "engine_launch.cuh"

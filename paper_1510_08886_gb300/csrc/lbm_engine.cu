@@ -4,9 +4,10 @@
 // (bundles of channels small enough to run a whole chunk in shared memory,
 // tiles of the others), CUDA-graph capture of a chunk of time steps plus the
 // per-solve reductions, and an autotuner of each velocity set's tile shape,
-// cells per tile and tiles per grab and of the persistent grid.  Storage fp64 (fp64 arithmetic), fp32, fp16 or bf16
-// (fp32 arithmetic); the device slot records are EngineSolve<double> for fp64
-// and EngineSolve<float> otherwise.
+// cells per tile and tiles per grab and of the persistent grid.  Storage fp64
+// (collision in 64-bit fixed point, fx64.cuh), fp32, fp16 or bf16 (fp32
+// arithmetic); the device slot records are EngineSolve<double> for fp64 and
+// EngineSolve<float> otherwise.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
