@@ -18,11 +18,15 @@
 //         unit U_G = 2 U, converted to fp64 (rounded to nearest) and relaxed
 //         with one fma: d* = (1 - omega) d + omega w G.
 //
-// Every rounding is to nearest or has zero mean: a bias of a fraction of a unit
-// per step would act on the flow like a body force.  Against a 113-bit reference
-// (random channel states, Kn 0.01 to 1, u 1e-3 to 3e-2) the rms error of a node's
-// post-collision moments relative to the FP64 evaluation's is 0.8 to 1.1 in the
-// density, 0.25 to 1.0 in x and 0.5 to 1.1 in y momentum.
+// Roundings are to nearest but for ties and for the low words that a product or a
+// shift drops, and a bias of a fraction of a unit per step acts on the flow like a
+// body force: over random channel states (Kn 0.01 to 1, u 1e-3 to 1e-2, Ma to 1e-2)
+// a node's mean error is up to 0.06 U_G in the density, 0.27 U_G in x and 0.09 U_G
+// in y momentum, against 0.09, 2.2 and 0.15 in fp64 arithmetic.  The rms error is
+// 0.17 to 0.78 of that of the same formulas in fp64 (tests/fx64/fx64_moments.cpp) and
+// 0.2 to 1.2 of that of the FP64 form (dp_collide), which shares sums between the
+// populations; in the first steps from rest, whose populations are far below the
+// force's scale, density and y momentum, both near zero there, are at up to 2.
 //
 // Per 32 nodes and step (D2V33, N = 4) this issues 3670 instructions, 33 of them
 // FP64, against ~475 FP64 ones of 64 cycles: 334 us per step on 4096 x 512 (1586),
@@ -727,7 +731,7 @@ inline Consts make_consts(double c_, double tau_, double dt_, double g_, int R, 
         (i ? k.th_exp : k.h_exp) = 62 - e;
     }
     // the rounding of the sums K enters the odd coefficients times theta c^4 e^3:
-    // harmless for theta < 1/8 (8 tau^2 c Ma: Kn up to 4 at Ma = 1e-3)
+    // below that of fp64 for theta < 1/8 (8 tau^2 c Ma: Kn up to 4 at Ma = 1e-3)
     if (k.emin > kLargestE || th >= 0.125L) k.ok = 0;
     k.c2 = to_mul(c * c, c2_point(emax), k.ok);
     k.h_63 = to_mul(h, 63, k.ok);

@@ -11,7 +11,7 @@ ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
 @pytest.mark.skipif(shutil.which("g++") is None, reason="no host compiler")
-@pytest.mark.parametrize("program", ["fx64_force", "fx64_rest", "fx64_rates", "fx64_range"])
+@pytest.mark.parametrize("program", ["fx64_force", "fx64_rest", "fx64_rates", "fx64_range", "fx64_moments"])
 def test_fixed_point_collision(program, tmp_path):
     exe = str(tmp_path / program)
     subprocess.run(["g++", "-O2", "-std=c++17", "-ffp-contract=off", "-Wno-unknown-pragmas",
