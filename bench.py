@@ -733,7 +733,7 @@ def main():
             "roofline": roofline,
             "cpu_baseline": cpu,
             "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": ncell * 8,
-                    "d2h_bytes_per_step": 4 * 8 + 4},
+                    "d2h_bytes_per_step": 256 + 4},
             "gpu_launches": launches,
             "clocks": clocks,
             "status": status, "mdot": mdot,
