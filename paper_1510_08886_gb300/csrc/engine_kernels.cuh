@@ -64,6 +64,10 @@ __device__ __forceinline__ void copy_params(const KParams<C>& src, KParams<C, MD
 }
 
 // emit: 0 = nothing, 1 = rho, u_x, u_y into the moment fields, 2 = u_x into prev
+// Resident blocks asked for in fp64: 4, 3 for more than 20 pairs, whose scratch and
+// constants leave no room for 5 (24 channels of 64 or 256 x 200 to 400, us per step at
+// 3 or 4 / 4 / 5: D2V16 141.7 / 141.6 / 136.7, D2V33 238.8 / 238.4 / 250.0, D2V32 262 / 262 /
+// 264, D2V48 410 / 409 / 416, D2V53 402 / 405 / 432).
 template <class SET, int N, typename S, typename C>
 __global__ void __launch_bounds__(kBlock, sizeof(C) == 8
                                               ? (SET::P > 20 ? 3 : 4)
@@ -77,6 +81,8 @@ k_engine_step(const EngineSolve<C>* __restrict__ solves, const EngineTile* __res
     __shared__ const S* sp[V];
     __shared__ S* dp[V];
     __shared__ int s_first[2];
+    // (the set's size only in fp64, where the full record is 17 KB: in fp32 the compact
+    // one's code spills 32 bytes instead of 16, 4 % slower on 40 channels)
     using Rec = KParams<C, sizeof(C) == 8 ? V : LBM_MAX_V>;
     __shared__ Rec s_k;
     const int ntiles = *ntiles_p;

@@ -48,6 +48,10 @@ using lbm::elem_bytes;
 
 namespace {
 
+// Fields and status in one copy up to this span: 18 us for 64 nodes, 22 us for 3000
+// (120 KB), against 46 to 48 us for four copies.  The span holds prev_ux besides and
+// goes through a host buffer that the solver keeps, hence the limit; at 48 us for
+// 12,000 nodes the four copies are still bound by the calls.
 constexpr size_t kSmallRead = 128 << 10;
 constexpr unsigned kStateMagic = 0x4c424d31u;   // "LBM1"
 
