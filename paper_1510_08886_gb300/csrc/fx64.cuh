@@ -28,9 +28,9 @@
 // populations; in the first steps from rest, whose populations are far below the
 // force's scale, density and y momentum, both near zero there, are at up to 2.
 //
-// Per 32 nodes and step (D2V33, N = 4) this issues 3670 instructions, 33 of them
-// FP64, against ~475 FP64 ones of 64 cycles: 334 us per step on 4096 x 512 (1586),
-// D2V16 163 us (12.8 GLUPS), D2V53 2048 x 512 303 us.
+// Per 32 nodes and step (D2V33, N = 4) this issues 3707 instructions, 34 of them
+// FP64, against ~475 FP64 ones of 64 cycles: 331 us per step on 4096 x 512 (1585 in
+// FP64), D2V16 166 us (816), D2V53 2048 x 512 293 us (1044).
 //
 // Nodes outside the range of the fixed-point form (a density far from 1, a flow
 // speed near the lattice's limit, non-finite values) and solves whose force

@@ -13,7 +13,7 @@
 //
 // Bound by one node's dependency chain: in fp64 ~700 integer instructions for the
 // coefficients on every lane, the sums over the lanes and the cluster barrier
-// (~370 cycles).  D2V16 1 x 64: 2.6 us per step (4.3 when ~100 FP64 instructions
+// (~370 cycles).  D2V16 1 x 64: 2.7 us per step (4.3 when ~100 FP64 instructions
 // of 64 cycles each made the chain); 1 x 600, 10 warps per CTA: 4.1 us against 6.0
 // with one launch per step; 1 x 1500, 24 warps: 6.7 against 6.0 (fp32: 2.2 against
 // 5.3).

@@ -1244,8 +1244,9 @@ __device__ __forceinline__ void wall_strip(const KParams<C, MV>& k, const S* src
 // fp64 copies them to shared memory as they arrive (cp.async) and runs the
 // fixed-point collision on them there (fx64.cuh), which leaves 96 registers and
 // 20 warps per SM.  fp32 is bound by HBM (D2V33 4096 x 512: 82 us per step, 6.7
-// TB/s), 16-bit by instruction issue, fp64 by integer issue and fetch (334 us,
-// 3.3 TB/s; 1586 us when the FP64 pipe evaluated it).
+// TB/s), 16-bit by latency and issue together at 29 warps per SM (fp16 64 us, 848 warp
+// instructions per 32 nodes, issue active 69 %), fp64 by integer issue and fetch (331
+// us, 3.35 TB/s, issue active 59 %; 1585 us when the FP64 pipe evaluated it).
 //  - fast path (block-uniform): the block's nodes lie in one row at least
 //    max|e_y| rows from both walls and max|e_x| columns from both ends, so
 //    every pull is a fixed offset from the node: one address per population;
